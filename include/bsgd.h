@@ -155,14 +155,17 @@ bsgd_status bsgd_forward_project(const bsgd_geometry *g, const void *x, bsgd_dty
  * bsgd_forward_project (Algorithm 1's BP step).
  *  r: device, batch * n_rows elements of type rt; rows outside the selected
  *     row blocks are not read.
- *  x: device, batch * n_cols float32 (BSGD_F32 only: the scatter accumulates
- *     with float atomics). With accumulate = 0 the voxels of the selected
+ *  x: device, batch * n_cols float32 (BSGD_F32 only: the sums are kept in
+ *     float). With accumulate = 0 the voxels of the selected
  *     column blocks are cleared first; other voxels are untouched.
- * Not bit-reproducible run to run (atomic order); results agree to float
- * rounding. For volumes, the views whose rays run mostly along x scatter into a
- * y-fastest float32 accumulator from the library's memory pool (n_cols floats),
- * added into x after each run of column blocks (x directly if the pool has no
- * room).
+ * Larger cone-beam volumes gather (the same sum in every run) from weights that
+ * the call lays out in the library's memory pool: n_views of the row blocks (at
+ * most 64 blocks at a time) * nu * (nv and some padding) floats. Otherwise, or
+ * if the pool has no room, the rays scatter: not bit-reproducible run to run
+ * (atomic order), results agree to float rounding; the views whose rays run
+ * mostly along x then scatter into a y-fastest float32 accumulator from the pool
+ * (n_cols floats), added into x after each run of column blocks (x directly if
+ * the pool has no room).
  */
 bsgd_status bsgd_back_project(const bsgd_geometry *g, const void *r, bsgd_dtype rt,
                               void *x, bsgd_dtype xt,

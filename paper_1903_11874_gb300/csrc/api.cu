@@ -121,10 +121,20 @@ extern "C" bsgd_status bsgd_back_project(const bsgd_geometry *g, const void *r, 
     BSGD_TRY(block_lists(g, row_blocks, n_rb, col_blocks, n_cb, rows, runs));
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t C = g->n_cols(), R = g->n_rows();
-    // y-fastest FP32 accumulator for the views whose rays run along x, added
-    // back into x after each run (optional, as in the forward projection)
-    float *gT = nullptr;
-    if (plain_wants_transpose(g, rows.data(), (int)rows.size()))
+    // the column form gathers from weights laid out row by row; where it is not
+    // taken (or there is no room for them) the views whose rays run along x
+    // scatter into a y-fastest FP32 accumulator, added back into x after each
+    // run (optional, as in the forward projection)
+    float *w = nullptr, *gT = nullptr;
+    int views = 0;
+    for (int i : rows) views += (int)g->block_views[i].size();
+    auto gathers = [&](const std::pair<int, int> &run) {
+        return column_bp_pays(g, g->plane_start[run.second] - g->plane_start[run.first], views);
+    };
+    const size_t W = std::any_of(runs.begin(), runs.end(), gathers) ? column_weights_len(g, std::min((int)rows.size(), 64)) : 0;
+    if (W) pool_try_alloc((void **)&w, W * 4, st);
+    if ((!w || !std::all_of(runs.begin(), runs.end(), gathers)) &&
+        plain_wants_transpose(g, rows.data(), (int)rows.size()))
         pool_try_alloc((void **)&gT, (size_t)C * 4, st);
     auto run_all = [&]() -> bsgd_status {
         for (int b = 0; b < batch; ++b) {
@@ -133,9 +143,13 @@ extern "C" bsgd_status bsgd_back_project(const bsgd_geometry *g, const void *r, 
             for (auto &run : runs) {
                 const int64_t v0 = (int64_t)g->plane_start[run.first] * g->dg.plane_stride;
                 const int64_t v1 = (int64_t)g->plane_start[run.second] * g->dg.plane_stride;
+                PlainLaunch L{rows.data(), (int)rows.size(), run.first, run.second, 0};
+                if (w && gathers(run)) {
+                    BSGD_TRY(launch_bp_column(g, L, rb, rt, xb, scale, accumulate, w, st));
+                    continue;
+                }
                 if (!accumulate) BSGD_CUDA(cudaMemsetAsync(xb + v0, 0, (v1 - v0) * 4, st));
                 if (gT) BSGD_CUDA(cudaMemsetAsync(gT + v0, 0, (v1 - v0) * 4, st));
-                PlainLaunch L{rows.data(), (int)rows.size(), run.first, run.second, 0};
                 BSGD_TRY(launch_bp_plain(g, L, rb, rt, xb, scale, st, gT));
                 if (gT) BSGD_TRY(plain_add_transposed(g, gT, xb, run.first, run.second, st));
             }
@@ -143,6 +157,7 @@ extern "C" bsgd_status bsgd_back_project(const bsgd_geometry *g, const void *r, 
         return BSGD_OK;
     };
     const bsgd_status s = run_all();
+    pool_free(w, st);
     pool_free(gT, st);
     return s;
 }

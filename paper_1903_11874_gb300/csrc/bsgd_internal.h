@@ -53,6 +53,14 @@ struct ViewRay {
 };
 static_assert(sizeof(ViewRay) == 64, "ViewRay is 4 x float4");
 
+// Line of one (view, detector column) of a cone beam in the xy plane: offsets
+// from the volume's centre where the ray parameter equals the rotation axis's
+// (high and low part), 1 / slope and slope per axis (column.cuh).
+struct ColRay {
+    float xh, xl, ix, dx;
+    float yh, yl, iy, dy;
+};
+
 // Detector rectangle [u0, u1] x [v0, v1] (inclusive; empty when u0 > u1).
 struct Band {
     int u0, u1, v0, v1;
@@ -79,6 +87,13 @@ struct DeviceGeom {
     int M, N, axis, max_views;
     int64_t n_rows, n_cols;
     int plane_stride;          // voxels per plane along the block axis
+    // Column form of a cone beam (column.cuh); cray is null where it is not used
+    const ColRay *cray;        // n_views x nu
+    float tc;                  // ray parameter of the rotation axis
+    float zs;                  // source height (voxels from the volume's low face)
+    float vstep;               // z slope per detector row
+    float vslack;              // rows (column.cuh, GatherVoxel)
+    int vpad, nvp;             // a row of weights: vpad zeros, nv values, zeros; nvp in all
 };
 
 }  // namespace bsgd
@@ -109,6 +124,7 @@ struct bsgd_geometry {
     int *d_view_block = nullptr;
     unsigned char *d_view_yfast = nullptr;
     int64_t *d_zoff = nullptr;
+    bsgd::ColRay *d_cray = nullptr;
     bsgd::DeviceGeom dg{};
     // Filled on first use by a solver state and kept for the geometry's life
     // (index: number of detector cells 1, 2 or 4): exact voxel-ray update
@@ -133,6 +149,12 @@ namespace bsgd {
 
 // ---------------------------------------------------------------------------
 // Projector launches (siddon.cu)
+
+// Selected row blocks of a plain launch (views = block_views of each).
+struct RowSel {
+    int n;
+    int ids[64];
+};
 
 enum TraceMode : int {
     kFpPlain = 0,   // y = (y or 0) + A x
@@ -173,6 +195,16 @@ bsgd_status plain_add_transposed(const bsgd_geometry *g, const float *gT, float 
                                  cudaStream_t st);
 bsgd_status launch_count(const bsgd_geometry *g, const PlainLaunch &L,
                          unsigned long long *d_count, cudaStream_t st);
+// Column form of the cone beam (column.cu). column_tables fills the geometry's
+// tables where the form applies; launch_bp_column back-projects by gathering,
+// from weights that it lays out row by row in `w` (column_weights_len floats; 0:
+// too many).
+bsgd_status column_tables(bsgd_geometry *g);
+bool column_bp_pays(const bsgd_geometry *g, int planes, int views);
+size_t column_weights_len(const bsgd_geometry *g, int n_rb);
+bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const void *r,
+                             bsgd_dtype rt, float *x, float scale, int accumulate, float *w,
+                             cudaStream_t st);
 // Clear the rows of every view of the listed row blocks.
 bsgd_status zero_rows(const bsgd_geometry *g, const int *row_ids, int n_rb, void *y,
                       bsgd_dtype yt, cudaStream_t st);
@@ -291,7 +323,6 @@ bsgd_status launch_fpbp_solve(const bsgd_geometry *g, const SolveDev &S, const v
                               bsgd_dtype st_t, int max_pairs, int max_tiles, cudaStream_t st);
 bsgd_status launch_count_cells(const bsgd_geometry *g, int j, int n_cells,
                                unsigned long long *d_counts, cudaStream_t st);
-
 }  // namespace bsgd
 
 namespace bsgd {

@@ -1,0 +1,177 @@
+// Column form of the circular cone beam: its tables and the back projection
+// that gathers (column.cuh).
+#include <algorithm>
+#include <cmath>
+
+#include "column.cuh"
+
+namespace bsgd {
+
+namespace {
+
+// Lines of every (view, detector column), from the FP32 ray table (the same rays
+// as the incremental walk's), in FP64.
+__global__ void column_tables_kernel(const DeviceGeom G, ColRay *__restrict__ cray) {
+    const int64_t n = (int64_t)G.n_views * G.nu;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const ViewRay &R = G.rays[k / G.nu];
+        const float fu = (float)(int)(k % G.nu) - 0.5f * (float)(G.nu - 1);
+        const float dx = fmaf(fu, R.cu[0], R.c0[0]) - R.p0[0], dy = fmaf(fu, R.cu[1], R.c0[1]) - R.p0[1];
+        const double X = (double)R.p0[0] + (double)G.tc * dx - 0.5 * G.nx;
+        const double Y = (double)R.p0[1] + (double)G.tc * dy - 0.5 * G.ny;
+        ColRay c;
+        c.xh = (float)X;
+        c.yh = (float)Y;
+        c.xl = (float)(X - c.xh);
+        c.yl = (float)(Y - c.yh);
+        c.dx = dx;
+        c.dy = dy;
+        c.ix = dx != 0.f ? (float)(1.0 / dx) : kFlat;
+        c.iy = dy != 0.f ? (float)(1.0 / dy) : kFlat;
+        // a line lying in a face belongs to the cell on its + side
+        if (dx == 0.f) c.xl += 1e-9f;
+        if (dy == 0.f) c.yl += 1e-9f;
+        cray[k] = c;
+    }
+}
+
+// w[slot][u][vpad + v] = scale * r[a][v][u] * |d| / (|j| ds): the ray's length
+// and the rise of its row j = v - (nv - 1) / 2 (the level row: j = 1), through a
+// 32 x 33 shared tile so that both sides are coalesced. Rows of nvp elements.
+template <typename T>
+__global__ void __launch_bounds__(256) column_weights_kernel(const DeviceGeom G, const RowSel R,
+                                                             const T *__restrict__ r, float scale,
+                                                             float *__restrict__ w) {
+    __shared__ float s[32][33];
+    const int a = sel_view(G, R, blockIdx.y);
+    if (a < 0) return;
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int tu = (G.nu + 31) / 32;
+    const int u0 = (blockIdx.x % tu) * 32, v0 = (int)(blockIdx.x / tu) * 32 - G.vpad;
+    const ColRay C = load_ray(G.cray + (size_t)a * G.nu + min(u0 + lane, G.nu - 1));
+    const float len = column_length2(G, C);
+#pragma unroll
+    for (int k = row; k < 32; k += 8) {
+        const int v = v0 + k, u = u0 + lane;
+        float val = 0.f;
+        if (v >= 0 && v < G.nv && u < G.nu)
+            val = ldf(r + ((int64_t)a * G.nv + v) * G.nu + u) * scale * column_weight(G, len, v);
+        s[k][lane] = val;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = row; k < 32; k += 8) {
+        const int u = u0 + k, v = v0 + lane;
+        if (u < G.nu && v + G.vpad < G.nvp) w[((size_t)blockIdx.y * G.nu + u) * G.nvp + v + G.vpad] = s[lane][k];
+    }
+}
+
+// The columns of a CTA: kGatherAcross along x, kGatherRows along y, one per warp.
+// out(index, value) for every voxel of planes [z0, z1), along x.
+template <class View, class Out>
+__device__ __forceinline__ void gather_cta(const DeviceGeom &G, int n_slots, View &&view, const float *__restrict__ w,
+                                           int z0, int z1, int n_cells, Out &&out) {
+    __shared__ GatherWarp warps[kGatherWarps];
+    const int tiles = (G.nx + kGatherAcross - 1) / kGatherAcross;
+    const int x0 = blockIdx.x % tiles * kGatherAcross, y0 = blockIdx.x / tiles * kGatherRows;
+    const int warp = threadIdx.x >> 5, x = x0 + warp % kGatherAcross, y = y0 + warp / kGatherAcross;
+    if (x < G.nx && y < G.ny) gather_column(G, n_slots, view, w, x, y, z0, z1, n_cells, warps[warp]);
+    __syncthreads();
+    for (int k = threadIdx.x; k < (z1 - z0) * kGatherWarps; k += blockDim.x) {
+        const int c = k % kGatherWarps, z = k / kGatherWarps, xx = x0 + c % kGatherAcross, yy = y0 + c / kGatherAcross;
+        if (xx < G.nx && yy < G.ny)
+            out(((int64_t)(z0 + z) * G.ny + yy) * G.nx + xx, warps[c].sums[z >> 5][z & 31]);
+    }
+}
+
+// x = (or +=) the plain back projection of planes [z0, z1), kGatherChunks chunks
+// of 32 per CTA (grid y).
+__global__ void __launch_bounds__(32 * kGatherWarps, 4)
+    bp_gather_kernel(const DeviceGeom G, const RowSel R, int z0, int z1, const float *__restrict__ w,
+                     float *__restrict__ x, int add) {
+    auto view = [&](int &slot, int &) {
+        const int k = R.n > 1 ? slot / G.max_views : 0;
+        return G.block_views[R.ids[k] * G.max_views + slot - k * G.max_views];
+    };
+    const int zb = z0 + (int)blockIdx.y * 32 * kGatherChunks;
+    gather_cta(G, R.n * G.max_views, view, w, zb, min(z1, zb + 32 * kGatherChunks), 1,
+               [&](int64_t k, float v) { x[k] = add ? x[k] + v : v; });
+}
+
+}  // namespace
+
+// Whether the back projection of `views` views into `planes` planes gathers. A
+// warp runs through all views of its column (0.43 us each, whatever the other
+// warps do), so small slabs seen from many views scatter instead: 64 x 64 x 32
+// from 360 views 151 us scattered, 164 gathered; 64^3 from 90 views 114 and 66
+// us; 48 x 48 x 32 from 24 views 35 and 23 us; 32^3 from 90 views 35 and 39 us.
+bool column_bp_pays(const bsgd_geometry *g, int planes, int views) {
+    const int64_t voxels = (int64_t)g->desc.nx * g->desc.ny * planes;
+    return g->dg.cray && voxels >= (views <= 32 ? 64000 : 160000);
+}
+
+bsgd_status column_tables(bsgd_geometry *g) {
+    const bsgd_geometry_desc &d = g->desc;
+    DeviceGeom &dg = g->dg;
+    if (d.kind != BSGD_CONE3D || d.nz < 2 || d.nv < 2) return BSGD_OK;
+    // rows more than two voxels apart at the axis: most voxels of a column meet
+    // no ray of a view, and the ray-driven scatter has less to do
+    if (d.dv * d.dso / d.dsd > 2.0 * d.dz) return BSGD_OK;
+    // rows are found by an addition that holds them in 22 bits
+    const double near = d.dso - 0.5 * std::hypot(d.nx * d.dx, d.ny * d.dy);
+    if (d.nv > (1 << 20) || d.dz * d.dsd / (near * d.dv) > 1e3) return BSGD_OK;
+    // a ray rises less than a voxel while it crosses a column
+    const double rise = 0.5 * (d.nv - 1) * d.dv / d.dz / d.dsd;   // voxels per mm along the axis
+    if (std::sqrt(2.0) * std::max(d.dx, d.dy) * rise > 0.95) return BSGD_OK;
+    dg.tc = (float)(d.dso / d.dsd);
+    dg.zs = g->rays[0].p0[2];
+    dg.vstep = g->rays[0].cv[2];
+    // rows that 32 planes can span past the first or last row that meets one of
+    // them: at the volume's near edge, with the change of a row's height in a cell
+    const double rows = d.dz * d.dsd / (near * d.dv);
+    const double change = rows * std::sqrt(2.0) * std::max(d.dx, d.dy) / near;   // rows per voxel of height
+    dg.vslack = (float)(32.0 * change * 1.01);
+    dg.vpad = (int)std::ceil(33.0 * rows + (2.0 * d.nz + 32.0) * change) + 8;
+    dg.nvp = (d.nv + 2 * dg.vpad + 7) / 8 * 8;
+    BSGD_CUDA(cudaMalloc((void **)&g->d_cray, sizeof(ColRay) * (size_t)d.n_views * d.nu));
+    const int64_t n = (int64_t)d.n_views * d.nu;
+    const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 152 * 16));
+    column_tables_kernel<<<gb, 128>>>(dg, g->d_cray);
+    BSGD_CUDA(cudaGetLastError());
+    BSGD_CUDA(cudaStreamSynchronize(0));
+    dg.cray = g->d_cray;
+    return BSGD_OK;
+}
+
+size_t column_weights_len(const bsgd_geometry *g, int n_rb) {
+    // rows of weights are addressed by 32-bit offsets
+    const size_t n = (size_t)n_rb * g->max_views * g->desc.nu * g->dg.nvp;
+    return n < (1ull << 32) ? n : 0;
+}
+
+static dim3 gather_grid(const bsgd_geometry *g, int planes, int z) {
+    const int across = (g->desc.nx + kGatherAcross - 1) / kGatherAcross, rows = (g->desc.ny + kGatherRows - 1) / kGatherRows;
+    return dim3((unsigned)(across * rows), (planes + 32 * kGatherChunks - 1) / (32 * kGatherChunks), z);
+}
+
+bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const void *r,
+                             bsgd_dtype rt, float *x, float scale, int accumulate, float *w,
+                             cudaStream_t st) {
+    const int z0 = g->plane_start[L.j0], z1 = g->plane_start[L.j1];
+    const dim3 grid = gather_grid(g, z1 - z0, 1);
+    for (int k = 0; k < L.n_rb; k += 64) {
+        RowSel R{};
+        R.n = std::min(64, L.n_rb - k);
+        for (int t = 0; t < R.n; ++t) R.ids[t] = L.row_ids[k + t];
+        const dim3 wg((unsigned)((g->desc.nu + 31) / 32 * ((g->dg.nvp + 31) / 32)), R.n * g->max_views);
+        if (rt == BSGD_F32) column_weights_kernel<float><<<wg, 256, 0, st>>>(g->dg, R, (const float *)r, scale, w);
+        else if (rt == BSGD_BF16) column_weights_kernel<__nv_bfloat16><<<wg, 256, 0, st>>>(g->dg, R, (const __nv_bfloat16 *)r, scale, w);
+        else column_weights_kernel<__half><<<wg, 256, 0, st>>>(g->dg, R, (const __half *)r, scale, w);
+        bp_gather_kernel<<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, R, z0, z1, w, x, accumulate || k > 0);
+        BSGD_CUDA(cudaGetLastError());
+    }
+    return BSGD_OK;
+}
+
+}  // namespace bsgd

@@ -243,6 +243,7 @@ static void free_geometry(bsgd_geometry *g) {
     cudaFree(g->d_view_block);
     cudaFree(g->d_view_yfast);
     cudaFree(g->d_zoff);
+    cudaFree(g->d_cray);
     for (int k = 0; k < 5; ++k) {
         cudaFree(g->d_counts[k]);
         cudaFree(g->d_cw[k]);
@@ -446,6 +447,10 @@ extern "C" bsgd_status bsgd_geometry_create(const bsgd_geometry_desc *desc, int 
     dg.n_rows = g->n_rows();
     dg.n_cols = g->n_cols();
     dg.plane_stride = g->axis == 2 ? d.nx * d.ny : d.nx;
+    if ((st = column_tables(g))) {
+        free_geometry(g);
+        return st;
+    }
     *out = g;
     return BSGD_OK;
 }

@@ -15,19 +15,6 @@
 
 namespace bsgd {
 
-// Selected row blocks of a plain launch (views = block_views of each).
-struct RowSel {
-    int n;
-    int ids[64];
-};
-
-__device__ __forceinline__ int sel_view(const DeviceGeom &G, const RowSel &R, int slot) {
-    const int k = slot / G.max_views, pos = slot % G.max_views;
-    if (k >= R.n) return -1;
-    const int i = R.ids[k];
-    return pos < G.block_nviews[i] ? G.block_views[i * G.max_views + pos] : -1;
-}
-
 // ---------------------------------------------------------------------------
 // Plain kernels
 

@@ -51,6 +51,13 @@ __device__ __forceinline__ int64_t zslot(const DeviceGeom &G, int j, int a, int 
     return G.zoff[(size_t)j * G.n_views + a] + (int64_t)(v - b.v0) * (b.u1 - b.u0 + 1) + (u - b.u0);
 }
 
+__device__ __forceinline__ int sel_view(const DeviceGeom &G, const RowSel &R, int slot) {
+    const int k = slot / G.max_views, pos = slot % G.max_views;
+    if (k >= R.n) return -1;
+    const int i = R.ids[k];
+    return pos < G.block_nviews[i] ? G.block_views[i * G.max_views + pos] : -1;
+}
+
 struct RayWalk {
     float tx, ty, tz;   // parameter left to the next interior plane per axis (INF: none)
     float te;           // parameter left to the exit face (INF until the exit axis has

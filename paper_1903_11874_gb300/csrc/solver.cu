@@ -1113,11 +1113,11 @@ bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int 
     const int64_t b0 = (int64_t)g->plane_start[j] * g->dg.plane_stride;
     const int64_t b1 = (int64_t)g->plane_start[j + 1] * g->dg.plane_stride;
     const int64_t n = g->n_cols(), m = g->n_rows();
-    float *v32 = nullptr, *w = nullptr, *y = nullptr, *vT = nullptr, *wT = nullptr;
+    float *v32 = nullptr, *w = nullptr, *y = nullptr, *vT = nullptr, *wT = nullptr, *cw = nullptr;
     double *v64 = nullptr, *nrm = nullptr;
     bsgd_status s = BSGD_OK;
     auto cleanup = [&]() {
-        for (void *p : {(void *)v32, (void *)w, (void *)y, (void *)v64, (void *)nrm, (void *)vT, (void *)wT})
+        for (void *p : {(void *)v32, (void *)w, (void *)y, (void *)v64, (void *)nrm, (void *)vT, (void *)wT, (void *)cw})
             pool_free(p, st);
     };
     if ((s = palloc((void **)&v32, n * 4, st)) || (s = palloc((void **)&w, n * 4, st)) ||
@@ -1132,13 +1132,18 @@ bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int 
         row_ids = all.data();
         n_rb = g->M;
     }
-    // y-fastest copies of v and of the BP accumulator for the views whose rays
-    // run along x (optional: without them the iteration is the same, slower)
-    if (plain_wants_transpose(g, row_ids, n_rb) &&
-        (!pool_try_alloc((void **)&vT, n * 4, st) || !pool_try_alloc((void **)&wT, n * 4, st))) {
-        pool_free(vT, st);
-        pool_free(wT, st);
-        vT = wT = nullptr;
+    // the column form's weights, or y-fastest copies for the views whose rays run
+    // along x: of the BP accumulator, and of v (optional: without them the
+    // iteration is the same, slower)
+    int views = 0;
+    for (int k = 0; k < n_rb; ++k) views += (int)g->block_views[row_ids[k]].size();
+    if (column_bp_pays(g, g->plane_start[j + 1] - g->plane_start[j], views)) {
+        const size_t W = column_weights_len(g, std::min(n_rb, 64));
+        if (W) pool_try_alloc((void **)&cw, W * 4, st);
+    }
+    if (plain_wants_transpose(g, row_ids, n_rb)) {
+        pool_try_alloc((void **)&vT, n * 4, st);
+        if (vT && !cw) pool_try_alloc((void **)&wT, n * 4, st);
     }
     PlainLaunch L{row_ids, n_rb, j, j + 1, 0};
     // A^T A v over block j: FP of v, then BP into w (and wT, added back)
@@ -1146,6 +1151,7 @@ bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int 
         BSGD_CUDA(cudaMemsetAsync(y, 0, m * 4, st));
         if (vT) BSGD_TRY(plain_transpose(g, v32, BSGD_F32, vT, j, j + 1, st));
         BSGD_TRY(launch_fp_plain(g, L, v32, BSGD_F32, y, BSGD_F32, 1, st, vT));
+        if (cw) return launch_bp_column(g, L, y, BSGD_F32, w, 1.0f, 0, cw, st);
         if (wT) BSGD_CUDA(cudaMemsetAsync(wT + b0, 0, (b1 - b0) * 4, st));
         BSGD_TRY(launch_bp_plain(g, L, y, BSGD_F32, w, 1.0f, st, wT));
         if (wT) BSGD_TRY(plain_add_transposed(g, wT, w, j, j + 1, st));
@@ -1589,6 +1595,7 @@ size_t state_bytes(const bsgd_geometry_desc &d, int M, int N, const bsgd_solve_p
     b += 4 * (size_t)65536 * stride;                   // trace
     b += 8 * (size_t)N * d.n_views * cells * (p.cells == BSGD_CELLS_GEOMETRIC ? 2 : 1);
     // geometry tables
+    if (d.kind == BSGD_CONE3D && d.nz > 1 && d.nv > 1) b += sizeof(ColRay) * (size_t)d.n_views * d.nu;
     b += 64 * (size_t)d.n_views + 16 * (size_t)d.n_views * (N + 1) + 4 * ((size_t)M * maxV + M + N + 1 + d.n_views);
     size_t t = 0;
     if (p.step_rule != BSGD_STEP_FIXED) t = std::max(t, C * 8 + R * 4 + C * 8 / N + 64);

@@ -1,0 +1,117 @@
+"""The gathering back projection of the cone beam (column.cu) against the FP64
+oracle, at the sizes where its pieces end: planes past a whole chunk of 32, an
+odd nz (the source's height inside a voxel), a level detector row, slabs on both
+sides of the source's height, detectors finer than half a voxel (more than one
+pair of rows per crossing) and coarser than one, columns past a CTA's tile,
+rays along the axes, 16-bit residuals."""
+import numpy as np
+import pytest
+
+from helpers import gpu_geom, oracle_geom, rel_l2
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import projector as P  # noqa: E402
+from paper_1903_11874_gb300 import binding as B  # noqa: E402
+from paper_1903_11874_gb300 import synth  # noqa: E402
+
+DEV = "cuda:0"
+
+
+def cone(nx, ny, nz, views, nu, nv, pitch, M=1, N=1, dso=200.0, dsd=400.0):
+    return dict(kind="cone3d", nx=nx, ny=ny, nz=nz, dx=1.0, dy=1.0, dz=1.0, n_views=views, nu=nu,
+                nv=nv, du=pitch, dv=pitch, dso=dso, dsd=dsd, M=M, N=N)
+
+
+CASES = {
+    "one_chunk_and_a_plane": cone(64, 61, 33, 8, 90, 70, 1.7),
+    "odd_height_level_row": cone(67, 64, 65, 8, 81, 91, 1.9),
+    "level_row_in_a_face": cone(64, 64, 64, 8, 80, 81, 2.1),
+    "fine_rows": cone(64, 64, 40, 4, 200, 150, 0.7),
+    "coarse_rows": cone(70, 66, 64, 16, 40, 40, 3.9),
+    "nine_chunks": cone(40, 40, 260, 4, 50, 120, 3.4),
+    "short_distance": cone(64, 64, 48, 8, 96, 64, 1.6, dso=80.0, dsd=200.0),
+    "rise_of_most_of_a_voxel": cone(48, 48, 72, 8, 60, 60, 3.2, dso=72.0, dsd=144.0),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_back_projection(name):
+    """Against the oracle, and against the scattering walk (thin blocks of planes
+    scatter), which runs on the same FP32 rays.
+
+    Bounds: a ray's ends are rounded to FP32 in voxels (up to 232 from the
+    volume's corner: 7.6e-6), which moves a face crossing by up to ~1.5e-5 voxel;
+    two crossings of a mean chord of 0.7 voxel: 4e-5 of the chord, against the
+    oracle. The walks share the rays, and the gather's own crossings carry
+    distances from the middle (<= 50 voxels, 1.9e-6): 2e-5 holds both."""
+    s = dict(CASES[name], N=CASES[name]["nz"] // 2)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = synth.normal_array(og.n_rows, 3).astype(np.float32)
+    rd = torch.from_numpy(r).to(DEV)
+    x = torch.full((og.n_cols,), 7.0, device=DEV)
+    B.bsgd_back_project(gg, rd, x)
+    got = x.cpu().double().numpy()
+    assert rel_l2(got, P.bp(og, r.astype(np.float64)).reshape(-1)) <= 4e-5
+    thin = torch.zeros_like(x)
+    for j in range(gg.N):
+        B.bsgd_back_project(gg, rd, thin, col_blocks=[j])
+    assert rel_l2(got, thin.cpu().double().numpy()) <= 2e-5
+    # the same sum in every run
+    again = torch.zeros_like(x)
+    B.bsgd_back_project(gg, rd, again)
+    assert torch.equal(x, again)
+
+
+def test_blocks_scale_accumulate_and_storage():
+    """Two separate runs of slabs (the middle one on both sides of the source's
+    height), some row blocks, added onto an image, from a BF16 residual."""
+    s = cone(72, 70, 160, 12, 90, 160, 1.9, M=4, N=5)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = torch.from_numpy(synth.normal_array(og.n_rows, 4)).to(DEV, torch.bfloat16)
+    base = synth.uniform_array(og.n_cols, 5).astype(np.float32)
+    x = torch.from_numpy(base).to(DEV)
+    B.bsgd_back_project(gg, r, x, row_blocks=[2, 0], col_blocks=[2, 4], scale=-0.5, accumulate=True)
+    rows = np.sort(np.concatenate([P.rows_of_views(og, P.row_block_views(og, 4, i)) for i in (0, 2)]))
+    r64 = r.double().cpu().numpy()
+    ref = base.astype(np.float64)
+    for j in (2, 4):
+        ref = ref - 0.5 * P.bp_rows(og, r64[rows], rows, P.column_block(og, 5, j))
+    got = x.cpu().double().numpy()
+    assert rel_l2(got, ref) <= 4e-5
+    untouched = np.concatenate([P.column_block_voxels(og, 5, j) for j in (0, 1, 3)])
+    assert np.array_equal(got[untouched], base[untouched])
+
+
+def near(mask, shape):
+    """The voxels of a mask and their neighbours along the axes and diagonals."""
+    m = np.pad(mask.reshape(shape), 1)
+    out = np.zeros_like(m)
+    for dz in (-1, 0, 1):
+        for dy in (-1, 0, 1):
+            for dx in (-1, 0, 1):
+                out |= np.roll(m, (dz, dy, dx), (0, 1, 2))
+    return out[1:-1, 1:-1, 1:-1].reshape(-1)
+
+
+def test_infinite_and_nan_weights_stay_on_their_rays():
+    """A NaN or infinite ray reaches the voxels it crosses, and none further off
+    than a corner it grazes within rounding."""
+    s = cone(64, 64, 64, 4, 80, 80, 2.1)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = np.zeros((4, 80, 80), dtype=np.float32)
+    r[1, 37, 40], r[2, 50, 20] = np.nan, np.inf
+    x = torch.zeros(og.n_cols, device=DEV)
+    B.bsgd_back_project(gg, torch.from_numpy(r.reshape(-1)).to(DEV), x)
+    got = x.cpu().numpy()
+    ray = np.zeros((4, 80, 80))
+    ray[1, 37, 40] = 1.0
+    a = P.bp(og, ray.reshape(-1)).reshape(-1)
+    ray[:] = 0.0
+    ray[2, 50, 20] = 1.0
+    b = P.bp(og, ray.reshape(-1)).reshape(-1)
+    near_a, near_b = near(a > 0, (64, 64, 64)), near(b > 0, (64, 64, 64))
+    assert np.all(np.isnan(got[a > 1e-3]))
+    assert np.all(np.isposinf(got[(b > 1e-3) & ~near_a]))
+    assert np.all(got[~near_a & ~near_b] == 0.0)
