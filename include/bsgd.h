@@ -330,6 +330,10 @@ typedef struct {
  * states (so a state per call costs no page mapping once the pool is warm); the
  * update counts and cell weights are computed once per geometry and kept with
  * it (destroy a geometry only after its states).
+ * A cone-beam state with slabs of 28 planes or more and enough voxels and views
+ * per iteration back-projects by gathering (see bsgd_back_project): it then
+ * holds the weights of an iteration's pairs (pairs * views per row block * nu *
+ * (nv and some padding) floats) in place of a y-fastest accumulator.
  * Errors: INVALID_ARG (alpha, gamma outside (0, 1], residual pair sampling with
  * more than one pair per iteration, n_cells not 2 (2D) or 4 (3D) with cells),
  * OOM, CUDA.
@@ -435,8 +439,10 @@ typedef enum {
     BSGD_STAGE_BP = 3,       /* back projection of the residual change        */
     BSGD_STAGE_UPDATE = 4,   /* x_J += mu g_J                                 */
     BSGD_STAGE_TV = 5,       /* TV proximal step (BSGD-TV)                    */
-    BSGD_STAGE_FPBP = 6,     /* FP, residual and BP in one kernel (1 to 4
-                                column blocks per iteration)                  */
+    BSGD_STAGE_FPBP = 6,     /* FP, residual and BP in one pass (1 to 4 column
+                                blocks per iteration), counted once: one
+                                kernel, or the FP with the residual and the
+                                gathering BP                                  */
     BSGD_N_STAGES = 7
 } bsgd_stage;
 
@@ -480,8 +486,9 @@ bsgd_status bsgd_state_read_profile(bsgd_state *s, bsgd_profile *out, void *stre
  * bsgd_state_restore: loads a checkpoint into s, a state created from the same
  *   geometry, parameters and y (a fresh one, or the same one to roll back);
  *   continue with bsgd_block_step and the x of the save. Restores the
- *   sampling mode the saved state ran with (bsgd_state_set_sampling).
- *   Synchronises `stream`. Errors: INVALID_ARG when the blob is not a
+ *   sampling mode the saved state ran with (bsgd_state_set_sampling). A blob of
+ *   a state that scattered (with a y-fastest part of g) restores into one that
+ *   gathers. Synchronises `stream`. Errors: INVALID_ARG when the blob is not a
  *   checkpoint of a state of this geometry, block counts, pair counts and
  *   storage type, or is truncated.
  */

@@ -202,6 +202,7 @@ bsgd_status launch_count(const bsgd_geometry *g, const PlainLaunch &L,
 bsgd_status column_tables(bsgd_geometry *g);
 bool column_bp_pays(const bsgd_geometry *g, int planes, int views);
 size_t column_weights_len(const bsgd_geometry *g, int n_rb);
+size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells);
 bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const void *r,
                              bsgd_dtype rt, float *x, float scale, int accumulate, float *w,
                              cudaStream_t st);
@@ -255,6 +256,9 @@ struct SolveDev {
     // adjacent addresses
     void *xT;          // image, [z][x][y], storage type
     float *gT;         // their part of the aggregated gradient, [z][x][y]
+    // Column form (column.cuh; null otherwise: no gT then, but xT): weights of the
+    // iteration's back projection, [pair][view of its row block][u][nvp]
+    float *w;
     double *eud;       // Algorithm 3: effective update direction of the window (or null)
     // owner-computes sharding: 1 for the column blocks this process owns; the
     // FP, BP and update of a pair whose block it does not own are skipped
@@ -323,6 +327,13 @@ bsgd_status launch_fpbp_solve(const bsgd_geometry *g, const SolveDev &S, const v
                               bsgd_dtype st_t, int max_pairs, int max_tiles, cudaStream_t st);
 bsgd_status launch_count_cells(const bsgd_geometry *g, int j, int n_cells,
                                unsigned long long *d_counts, cudaStream_t st);
+// Column form (column.cu): the weights r - r~^j of every drawn pair (and r~^j =
+// r) where no FP pass left them, and the back projection of the drawn pairs into
+// g by gathering.
+bsgd_status launch_column_change(const bsgd_geometry *g, const SolveDev &S, bsgd_dtype st_t,
+                                 int max_pairs, cudaStream_t st);
+bsgd_status launch_column_solve(const bsgd_geometry *g, const SolveDev &S, int max_cols, cudaStream_t st);
+
 }  // namespace bsgd
 
 namespace bsgd {
@@ -390,6 +401,9 @@ __host__ __device__ inline bool round_skips(int period, unsigned long long round
     return period > 1 && round % (unsigned long long)period != 0;
 }
 
+// bsgd_state_create; column: take the column form where the geometry has it.
+bsgd_status state_create(const bsgd_geometry *g, const bsgd_solve_params *p, const void *y, bsgd_dtype yt,
+                         bool column, cudaStream_t st, bsgd_state **out);
 // Fill a request descriptor from a live state (solver.cu).
 bsgd_status state_descriptor(const bsgd_state *s, void *x, ReqDesc *out);
 bsgd_status state_first_draw(bsgd_state *s, cudaStream_t st);

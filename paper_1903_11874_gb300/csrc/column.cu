@@ -99,6 +99,79 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 4)
                [&](int64_t k, float v) { x[k] = add ? x[k] + v : v; });
 }
 
+// g_J += (A_R^J)^T w over the drawn pairs of column block J (blockIdx.z of the
+// iteration's blocks).
+__global__ void __launch_bounds__(32 * kGatherWarps, 4) solve_gather_kernel(const DeviceGeom G, const SolveDev S) {
+    __shared__ int s_pairs[kMaxPairs];
+    const Work &W = *S.work;
+    if ((int)blockIdx.z >= W.n_cols) return;
+    const int j = W.cols[blockIdx.z];
+    if (S.owned && !S.owned[j]) return;   // another process owns block j
+    const int z1 = G.plane_start[j + 1], zb = G.plane_start[j] + (int)blockIdx.y * 32 * kGatherChunks;
+    if (zb >= z1) return;
+    int np = 0;   // pairs of this block (the same in every thread)
+    for (int p = 0; p < W.n_pairs; ++p)
+        if (W.pair_j[p] == j) {
+            if (threadIdx.x == 0) s_pairs[np] = p;
+            ++np;
+        }
+    __syncthreads();
+    auto view = [&](int &slot, int &cell) {   // slot: of the pairs' views, then of the weights
+        const int k = np > 1 ? slot / G.max_views : 0, s = slot - k * G.max_views, p = s_pairs[k];
+        slot = p * G.max_views + s;
+        if (S.n_cells > 1) cell = S.cells[slot];
+        return G.block_views[W.pair_i[p] * G.max_views + s];
+    };
+    gather_cta(G, np * G.max_views, view, S.w, zb, min(z1, zb + 32 * kGatherChunks), S.n_cells,
+               [&](int64_t k, float v) { S.g[k] += v; });
+}
+
+// The weights of pair blockIdx.z at view slot blockIdx.y, over a 32 x 32 tile of
+// its band: r - r~^j for the rays that take part (r~^j = r), 0 for the others.
+template <typename T>
+__global__ void __launch_bounds__(256) column_change_kernel(const DeviceGeom G, const SolveDev S) {
+    __shared__ float s[32][33];
+    const Work &W = *S.work;
+    const int p = blockIdx.z, slot = blockIdx.y;
+    if (p >= W.n_pairs) return;
+    const int i = W.pair_i[p], j = W.pair_j[p];
+    if (S.owned && !S.owned[j]) return;   // another process owns block j
+    if (slot >= G.block_nviews[i]) return;
+    const int a = G.block_views[i * G.max_views + slot];
+    const Band b = G.bands[(size_t)a * (G.N + 1) + j];
+    if (b.u0 > b.u1 || b.v0 > b.v1) return;
+    const int tu = (b.u1 - b.u0 + 32) / 32;
+    const int u0 = b.u0 + (int)(blockIdx.x % tu) * 32, v0 = b.v0 + (int)(blockIdx.x / tu) * 32;
+    if (v0 > b.v1) return;
+    Band c = b;   // the rays of the drawn cell
+    if (S.n_cells > 1) cell_rect(G.nu, G.nv, S.n_cells, S.cells[p * G.max_views + slot], c);
+    const T *r = reinterpret_cast<const T *>(S.r);
+    T *rt = reinterpret_cast<T *>(S.rt);
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const ColRay C = load_ray(G.cray + (size_t)a * G.nu + min(u0 + lane, G.nu - 1));
+    const float len = column_length2(G, C);
+#pragma unroll
+    for (int k = row; k < 32; k += 8) {
+        const int u = u0 + lane, v = v0 + k;
+        float dw = 0.f;
+        if (u >= c.u0 && u <= c.u1 && v >= c.v0 && v <= c.v1) {
+            bool in;
+            const int64_t kt = zslot(G, j, a, u, v, in);
+            const float rv = ldv(r + ((int64_t)a * G.nv + v) * G.nu + u);
+            dw = (rv - ldv(rt + kt)) * column_weight(G, len, v);
+            stf(rt + kt, rv);
+        }
+        s[k][lane] = dw;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = row; k < 32; k += 8) {
+        const int u = u0 + k, v = v0 + lane;
+        if (u <= b.u1 && v <= b.v1)
+            S.w[(((int64_t)p * G.max_views + slot) * G.nu + u) * G.nvp + G.vpad + v] = s[lane][k];
+    }
+}
+
 }  // namespace
 
 // Whether the back projection of `views` views into `planes` planes gathers. A
@@ -171,6 +244,43 @@ bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const
         bp_gather_kernel<<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, R, z0, z1, w, x, accumulate || k > 0);
         BSGD_CUDA(cudaGetLastError());
     }
+    return BSGD_OK;
+}
+
+// Floats of the weights of a solver that draws kM row blocks and kN column blocks
+// per iteration, 0 where its BP scatters beside the FP in one pass instead. That
+// pass sets a ray up once for both, so the gather needs full warps (slabs of 28
+// planes or more) and enough columns and views to pay for a pass of its own:
+// us per iteration scattered / gathered (FP32, 8 or 4 row blocks), one block:
+// 256^2 x 32 from 45 views 432 / 390, 192^2 x 32 from 22 160 / 148, 96^2 x 32
+// from 45 83 / 81, 256^2 x 32 from 11 162 / 169, 256^2 x 16 from 45 258 / 312;
+// two blocks: 256^2 x 32 from 45 887 / 758, 128^2 x 32 from 11 120 / 90, 96^2 x
+// 12 from 22 70 / 68.
+// With detector cells one block's pass traces a fraction of the rays that the
+// gather lists: 160^2 x 32 from 45 views 90 / 109, 256^2 x 32 258 / 260.
+size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells) {
+    if (!g->dg.cray || (cells && kN == 1)) return 0;
+    const int planes = g->desc.nz / g->N;   // of the thinnest slab
+    const int64_t work = (int64_t)g->desc.nx * g->desc.ny * planes * kN * g->max_views * kM;
+    if (planes < 28 || work < (kN > 1 ? 10000000 : 25000000)) return 0;
+    return column_weights_len(g, kM * kN);
+}
+
+bsgd_status launch_column_change(const bsgd_geometry *g, const SolveDev &S, bsgd_dtype st_t,
+                                 int max_pairs, cudaStream_t st) {
+    const dim3 grid((unsigned)((g->desc.nu + 31) / 32 * ((g->desc.nv + 31) / 32)), g->max_views, max_pairs);
+    if (st_t == BSGD_F32) column_change_kernel<float><<<grid, 256, 0, st>>>(g->dg, S);
+    else if (st_t == BSGD_BF16) column_change_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->dg, S);
+    else column_change_kernel<__half><<<grid, 256, 0, st>>>(g->dg, S);
+    BSGD_CUDA(cudaGetLastError());
+    return BSGD_OK;
+}
+
+bsgd_status launch_column_solve(const bsgd_geometry *g, const SolveDev &S, int max_cols, cudaStream_t st) {
+    int planes = 1;
+    for (int j = 0; j < g->N; ++j) planes = std::max(planes, g->plane_start[j + 1] - g->plane_start[j]);
+    solve_gather_kernel<<<gather_grid(g, planes, max_cols), 32 * kGatherWarps, 0, st>>>(g->dg, S);
+    BSGD_CUDA(cudaGetLastError());
     return BSGD_OK;
 }
 

@@ -297,7 +297,7 @@ bsgd_status admit_one(bsgd_server *S, Request *r, cudaStream_t stream) {
     BSGD_TRY(pool_alloc(&dy, R * ys, stream));
     cudaError_t e = cudaMemcpyAsync(dy, r->y.data(), R * ys, cudaMemcpyHostToDevice, stream);
     bsgd_status st = e == cudaSuccess ? BSGD_OK : cuda_fail(e, "copy of y");
-    if (!st) st = bsgd_state_create(r->g, &prm, dy, r->yt, stream, &r->st);
+    if (!st) st = state_create(r->g, &prm, dy, r->yt, false, stream, &r->st);
     cudaStreamSynchronize(stream);
     pool_free(dy, stream);
     BSGD_TRY(st);

@@ -11,7 +11,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "siddon_device.cuh"
+#include "column.cuh"
 
 namespace bsgd {
 
@@ -164,7 +164,7 @@ __global__ void zero_views_kernel(const DeviceGeom G, const RowSel R, void *y, i
 
 __device__ __forceinline__ bool solve_pixel(const DeviceGeom &G, const SolveDev &S, int tile,
                                             int slot, int p, int &a, int &i, int &j, int &u,
-                                            int &v, bool &in_band) {
+                                            int &v, bool &in_band, bool whole = false) {
     const Work &W = *S.work;
     if (p >= W.n_pairs) return false;
     i = W.pair_i[p];
@@ -172,7 +172,7 @@ __device__ __forceinline__ bool solve_pixel(const DeviceGeom &G, const SolveDev 
     if (slot >= G.block_nviews[i]) return false;
     a = G.block_views[i * G.max_views + slot];
     Band b = G.bands[(size_t)a * (G.N + 1) + j];
-    if (S.n_cells > 1) cell_rect(G.nu, G.nv, S.n_cells, S.cells[p * G.max_views + slot], b);
+    if (!whole && S.n_cells > 1) cell_rect(G.nu, G.nv, S.n_cells, S.cells[p * G.max_views + slot], b);
     int nt;
     in_band = G.nv > 1 ? tile_pixel<true>(b, tile, u, v, nt) : tile_pixel<false>(b, tile, u, v, nt);
     return tile < nt;
@@ -258,15 +258,40 @@ __device__ __forceinline__ void bp_solve_body(const DeviceGeom &G, const SolveDe
     });
 }
 
+// Whether ray (u, v) takes part in the pair whose drawn cell is at cells[k].
+__device__ __forceinline__ bool in_cell(const DeviceGeom &G, const SolveDev &S, int k, int u, int v) {
+    if (S.n_cells <= 1) return true;
+    const int cell = S.cells[k];
+    return cell < 0 || (((cell & 1) != 0) == (u >= G.nu / 2) &&
+                        (S.n_cells != 4 || ((cell >> 1) != 0) == (v >= G.nv / 2)));
+}
+
+// Weight of ray (u, v) for the gathering back projection (0 for a ray of the
+// band that takes no part). A store per ray into a column of nvp: turning a
+// CTA's tile through shared memory first made the pass slower (176-199 against
+// 165-180 us on the 256^3 workload: its barriers hold a CTA's short rays until
+// the longest is done).
+__device__ __forceinline__ void put_weight(const DeviceGeom &G, const SolveDev &S, int64_t view_slot, int a,
+                                           int u, int v, float dw) {
+    if (dw != 0.f) {
+        const ColRay C = load_ray(G.cray + (size_t)a * G.nu + u);
+        dw *= column_weight(G, column_length2(G, C), v);
+    }
+    S.w[(view_slot * G.nu + u) * G.nvp + G.vpad + v] = dw;
+}
+
 // FP, residual and BP of one ray in one pass (one column block per iteration):
 // the ray's BP weight r_new - r~ depends only on its own FP, so the back
-// projection follows the forward walk without waiting for other rays.
-template <typename T>
+// projection follows the forward walk without waiting for other rays. kGather:
+// the weight is left for the gathering back projection instead.
+template <typename T, bool kGather>
 __device__ __forceinline__ void fpbp_solve_body(const DeviceGeom &G, const SolveDev &S,
                                                 const T *__restrict__ x, int tile, int slot, int p) {
     int a, i, j, u, v;
     bool act;
-    if (!solve_pixel(G, S, tile, slot, p, a, i, j, u, v, act)) return;
+    if (!solve_pixel(G, S, tile, slot, p, a, i, j, u, v, act, kGather)) return;
+    const bool band = act;
+    if (kGather) act = act && in_cell(G, S, p * G.max_views + slot, u, v);
     const int plo = G.plane_start[j], phi = G.plane_start[j + 1];
     const bool yf = act && S.xT != nullptr && G.view_yfast[a];
     float zn = 0.f;
@@ -307,7 +332,12 @@ __device__ __forceinline__ void fpbp_solve_body(const DeviceGeom &G, const Solve
         stf(rt + kj, rn);
     }
     for (int o = 16; o > 0; o >>= 1) dn += __shfl_xor_sync(0xffffffffu, dn, o);
-    if ((threadIdx.x & 31) == 0 && act && dn != 0.0) atomicAdd(S.S + (size_t)i * G.nv + v, dn);
+    // lane 0 has the lowest u, so it is in the band whenever any lane is
+    if ((threadIdx.x & 31) == 0 && band && dn != 0.0) atomicAdd(S.S + (size_t)i * G.nv + v, dn);
+    if (kGather) {
+        if (band) put_weight(G, S, (int64_t)p * G.max_views + slot, a, u, v, dw);
+        return;
+    }
     if (!act || dw == 0.f) return;
     float *dst = (S.gT != nullptr && G.view_yfast[a]) ? S.gT : S.g;
     RayWalk w;
@@ -318,10 +348,10 @@ __device__ __forceinline__ void fpbp_solve_body(const DeviceGeom &G, const Solve
     });
 }
 
-template <typename T>
+template <typename T, bool kGather>
 __global__ void __launch_bounds__(128) fpbp_solve_kernel(const DeviceGeom G, const SolveDev S,
                                                          const T *__restrict__ x) {
-    fpbp_solve_body<T>(G, S, x, blockIdx.x / G.max_views, blockIdx.x % G.max_views, blockIdx.z);
+    fpbp_solve_body<T, kGather>(G, S, x, blockIdx.x / G.max_views, blockIdx.x % G.max_views, blockIdx.z);
 }
 
 // FP, residual and BP of one ray in one pass when an iteration selects several
@@ -333,7 +363,7 @@ __global__ void __launch_bounds__(128) fpbp_solve_kernel(const DeviceGeom G, con
 // for that pair; the others keep their z^j and r~^j. The work item is a tile
 // of the bounding box of the selected blocks' bands (the rows the split path's
 // residual pass covers) for one view of one selected row block (rs).
-template <typename T, int NC>
+template <typename T, int NC, bool kGather>
 __device__ __forceinline__ void fpbpm_solve_body(const DeviceGeom &G, const SolveDev &S,
                                                  const T *__restrict__ x, int tile, int slot,
                                                  int rs) {
@@ -375,12 +405,7 @@ __device__ __forceinline__ void fpbpm_solve_body(const DeviceGeom &G, const Solv
         // outside it) and in the detector cell drawn for the pair at this view
         // (pairs are the drawn rows x the drawn columns, row-major)
         part[c] = inb[c];
-        if (part[c] && S.n_cells > 1) {
-            const int cell = S.cells[(rs * W.n_cols + c) * G.max_views + slot];
-            if (cell >= 0)
-                part[c] = ((cell & 1) != 0) == (u >= G.nu / 2) &&
-                          (S.n_cells != 4 || ((cell >> 1) != 0) == (v >= G.nv / 2));
-        }
+        if (part[c]) part[c] = in_cell(G, S, (rs * W.n_cols + c) * G.max_views + slot, u, v);
         if (!part[c]) continue;
         RayWalk w;
         if (ray_setup(G, a, u, v, G.plane_start[js[c]], G.plane_start[js[c] + 1], w, yf)) {
@@ -430,6 +455,19 @@ __device__ __forceinline__ void fpbpm_solve_body(const DeviceGeom &G, const Solv
     const bool yb = S.gT != nullptr && G.view_yfast[a];
     float *dst = yb ? S.gT : S.g;
     T *rt = reinterpret_cast<T *>(S.rt);
+    if (kGather) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            if (!act || !inb[c]) continue;
+            float dw = 0.f;
+            if (part[c]) {
+                dw = rn - ldv(rt + kj[c]);
+                stf(rt + kj[c], rn);
+            }
+            put_weight(G, S, (int64_t)(rs * W.n_cols + c) * G.max_views + slot, a, u, v, dw);
+        }
+        return;
+    }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         if (!act || !part[c]) continue;
@@ -445,10 +483,10 @@ __device__ __forceinline__ void fpbpm_solve_body(const DeviceGeom &G, const Solv
     }
 }
 
-template <typename T, int NC>
+template <typename T, int NC, bool kGather>
 __global__ void __launch_bounds__(128) fpbpm_solve_kernel(const DeviceGeom G, const SolveDev S,
                                                           const T *__restrict__ x) {
-    fpbpm_solve_body<T, NC>(G, S, x, blockIdx.x / G.max_views, blockIdx.x % G.max_views, blockIdx.z);
+    fpbpm_solve_body<T, NC, kGather>(G, S, x, blockIdx.x / G.max_views, blockIdx.x % G.max_views, blockIdx.z);
 }
 
 template <typename T, bool FUSED>
@@ -596,9 +634,9 @@ __global__ void __launch_bounds__(128, CT ? 1 : (MULTI ? 7 : 10))
             const int tile = (int)(local % q.max_tiles);
             const int p = (int)(local / q.max_tiles);
             const T *x = reinterpret_cast<const T *>(q.x);
-            if (!MULTI) fpbp_solve_body<T>(q.G, q.S, x, tile, slot, p);
-            else if (q.kN <= 2) fpbpm_solve_body<T, 2>(q.G, q.S, x, tile, slot, p);
-            else fpbpm_solve_body<T, 4>(q.G, q.S, x, tile, slot, p);
+            if (!MULTI) fpbp_solve_body<T, false>(q.G, q.S, x, tile, slot, p);
+            else if (q.kN <= 2) fpbpm_solve_body<T, 2, false>(q.G, q.S, x, tile, slot, p);
+            else fpbpm_solve_body<T, 4, false>(q.G, q.S, x, tile, slot, p);
             continue;
         }
         const int e = round_entry(T_, lo, hi, item);
@@ -621,9 +659,9 @@ __global__ void __launch_bounds__(128, CT ? 1 : (MULTI ? 7 : 10))
         local /= sG.max_views;
         const int tile = (int)(local % max_tiles);
         const int p = (int)(local / max_tiles);   // pair (one block) or row-block slot
-        if (!MULTI) fpbp_solve_body<T>(sG, sS, x, tile, slot, p);
-        else if (kN <= 2) fpbpm_solve_body<T, 2>(sG, sS, x, tile, slot, p);
-        else fpbpm_solve_body<T, 4>(sG, sS, x, tile, slot, p);
+        if (!MULTI) fpbp_solve_body<T, false>(sG, sS, x, tile, slot, p);
+        else if (kN <= 2) fpbpm_solve_body<T, 2, false>(sG, sS, x, tile, slot, p);
+        else fpbpm_solve_body<T, 4, false>(sG, sS, x, tile, slot, p);
     }
 }
 
@@ -857,9 +895,13 @@ bsgd_status launch_fpbp_solve(const bsgd_geometry *g, const SolveDev &S, const v
     // view slot fastest: CTAs running together hold the same band rows of
     // every view, and a launch ends on the band's last (edge) rows
     dim3 grid((unsigned)max_tiles * g->max_views, 1, max_pairs);
-    if (st_t == BSGD_F32) fpbp_solve_kernel<float><<<grid, 128, 0, st>>>(g->dg, S, (const float *)x);
-    else if (st_t == BSGD_BF16) fpbp_solve_kernel<__nv_bfloat16><<<grid, 128, 0, st>>>(g->dg, S, (const __nv_bfloat16 *)x);
-    else fpbp_solve_kernel<__half><<<grid, 128, 0, st>>>(g->dg, S, (const __half *)x);
+#define FPBP_GO(T)                                                                              \
+    if (S.w) fpbp_solve_kernel<T, true><<<grid, 128, 0, st>>>(g->dg, S, (const T *)x);          \
+    else fpbp_solve_kernel<T, false><<<grid, 128, 0, st>>>(g->dg, S, (const T *)x);
+    if (st_t == BSGD_F32) { FPBP_GO(float) }
+    else if (st_t == BSGD_BF16) { FPBP_GO(__nv_bfloat16) }
+    else { FPBP_GO(__half) }
+#undef FPBP_GO
     BSGD_CUDA(cudaGetLastError());
     return BSGD_OK;
 }
@@ -871,7 +913,9 @@ bsgd_status launch_fpbpm_solve(const bsgd_geometry *g, const SolveDev &S, const 
         return fail(BSGD_ERR_INVALID_ARG, "fused multi-block pass takes 2 to 4 column blocks");
     // view slot fastest, as in the one-block fused kernel
     dim3 grid((unsigned)max_tiles * g->max_views, 1, max_rows);
-#define FPBPM_GO(T, NC) fpbpm_solve_kernel<T, NC><<<grid, 128, 0, st>>>(g->dg, S, (const T *)x);
+#define FPBPM_GO(T, NC)                                                                          \
+    if (S.w) fpbpm_solve_kernel<T, NC, true><<<grid, 128, 0, st>>>(g->dg, S, (const T *)x);     \
+    else fpbpm_solve_kernel<T, NC, false><<<grid, 128, 0, st>>>(g->dg, S, (const T *)x);
 #define FPBPM_T(T) if (n_cols <= 2) { FPBPM_GO(T, 2) } else { FPBPM_GO(T, 4) }
     if (st_t == BSGD_F32) { FPBPM_T(float) }
     else if (st_t == BSGD_BF16) { FPBPM_T(__nv_bfloat16) }

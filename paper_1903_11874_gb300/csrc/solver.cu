@@ -8,6 +8,9 @@
 //   residual_kernel   only when several column blocks share a row block
 //   bp_solve_kernel   g_J += (A_R^J)^T (r_R - r~^J_R), r~^J_R = r_R (siddon.cu)
 //   update_kernel     x_J += mu g_J
+// With one to four column blocks per iteration the three passes in between are
+// one kernel (siddon.cu), or, where the BP gathers (column.cu), an FP with the
+// residual that leaves the weights r_R - r~^J_R and the gather.
 // The snapshot r~^J equals keeping Algorithm 1's memory g-hat^i: it stores the
 // residual the last BP of (i, J) used, so the BP of the change replaces
 // g-hat^i_J by the new one exactly.
@@ -16,7 +19,7 @@
 #include <cstring>
 #include <map>
 
-#include "siddon_device.cuh"
+#include "column.cuh"
 
 namespace bsgd {
 
@@ -510,7 +513,7 @@ __device__ __forceinline__ float updated(const T *x, const T *xlo, int64_t k, fl
 // Work of column block c of the iteration, shared by `nblk` CTAs of 256 threads
 // (this one is `blk`). Without the y-fastest copies: a strided pass over the
 // slab. With them: 32 x 32 (y, x) tiles of each z plane, where the gradient is
-// g + transpose(gT) and the new x is also written transposed into xT, both
+// g + transpose(gT) (g alone where the BP gathers) and the new x is also written transposed into xT, both
 // transposes staged through shared memory so every global access is coalesced.
 template <typename T>
 __device__ void update_body(const DeviceGeom &G, const SolveDev &S, T *__restrict__ x,
@@ -520,7 +523,7 @@ __device__ void update_body(const DeviceGeom &G, const SolveDev &S, T *__restric
     const int j = W.cols[c];
     if (S.owned && !S.owned[j]) return;   // another process owns block j
     const float mu = (float)*S.mu;
-    if (S.gT == nullptr) {
+    if (S.xT == nullptr) {
         const int64_t b0 = (int64_t)G.plane_start[j] * G.plane_stride;
         const int64_t b1 = (int64_t)G.plane_start[j + 1] * G.plane_stride;
         for (int64_t k = b0 + (int64_t)blk * blockDim.x + threadIdx.x; k < b1;
@@ -554,7 +557,7 @@ __device__ void update_body(const DeviceGeom &G, const SolveDev &S, T *__restric
         for (int q = 0; q < 4; ++q) {
             const int k = row + 8 * q;
             const bool inT = full || (x0 + k < nx && y0 + lane < ny);   // gT rows: fixed x
-            gt[q] = inT ? S.gT[bT + k * ny + lane] : 0.f;
+            gt[q] = inT && S.gT ? S.gT[bT + k * ny + lane] : 0.f;
             const bool inX = full || (y0 + k < ny && x0 + lane < nx);   // x rows: fixed y
             const int64_t idx = bX + k * nx + lane;
             gv[q] = inX ? S.g[idx] : 0.f;
@@ -923,6 +926,7 @@ struct bsgd_state {
     void *xlo = nullptr;        // low-order image term (16-bit storage only)
     void *xT = nullptr;         // y-fastest copy of x (volumes only)
     float *gT = nullptr;        // y-fastest part of g (volumes only)
+    float *w = nullptr;         // column form: weights of an iteration's BP (then no gT)
     float *grad = nullptr;
     double *S = nullptr, *cw = nullptr, *d_mu = nullptr;
     Work *work = nullptr;
@@ -1052,7 +1056,7 @@ void pool_free(void *p, cudaStream_t st) {
 static void free_state(bsgd_state *s) {
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
     // counts and cw belong to the geometry's cache; replay is a plain allocation
-    void *ptrs[] = {s->y, s->z, s->rt, s->r, s->xlo, s->xT, s->gT, s->grad, s->S, s->d_mu, s->work, s->cells,
+    void *ptrs[] = {s->y, s->z, s->rt, s->r, s->xlo, s->xT, s->gT, s->w, s->grad, s->S, s->d_mu, s->work, s->cells,
                     s->wband, s->d_iter, s->x0_flag, s->owned, s->wscratch, s->ticket, s->trace,
                     s->updates, s->pair_upd, s->eud, s->eud_prev, s->am_part, s->am};
     for (void *p : ptrs) pfree(p);
@@ -1303,12 +1307,16 @@ static bsgd_status geometry_tables(const bsgd_geometry *g, int n_cells, bool wei
 extern "C" bsgd_status bsgd_state_create(const bsgd_geometry *g, const bsgd_solve_params *p,
                                          const void *y, bsgd_dtype yt, void *stream,
                                          bsgd_state **out) {
+    return state_create(g, p, y, yt, true, (cudaStream_t)stream, out);
+}
+
+bsgd_status bsgd::state_create(const bsgd_geometry *g, const bsgd_solve_params *p, const void *y,
+                               bsgd_dtype yt, bool column, cudaStream_t st, bsgd_state **out) {
     if (!g || !p || !y || !out) return fail(BSGD_ERR_INVALID_ARG, "NULL argument");
     *out = nullptr;
     if (!dtype_ok(yt)) return fail(BSGD_ERR_INVALID_ARG, "bad y dtype");
     BSGD_TRY(check_params(g, p));
     BSGD_TRY(check_device(g));
-    cudaStream_t st = (cudaStream_t)stream;
     bsgd_state *s = new (std::nothrow) bsgd_state();
     if (!s) return fail(BSGD_ERR_OOM, "host allocation failed");
     s->g = g;
@@ -1335,6 +1343,10 @@ extern "C" bsgd_status bsgd_state_create(const bsgd_geometry *g, const bsgd_solv
     const int N = g->N, M = g->M, V = g->desc.n_views;
     bsgd_status e = BSGD_OK;
     const int64_t Z = g->zlen;   // compact band storage of z^j and r~^j
+    // column form: the BP gathers from weights that the FP leaves; without room
+    // for them the state scatters
+    const size_t W = column ? column_solve_len(g, s->kM, s->kN, p->cells != BSGD_CELLS_NONE) : 0;
+    if (W) pool_try_alloc((void **)&s->w, W * 4, st);
     if ((e = palloc(&s->y, R * es, st)) || (e = palloc(&s->z, (size_t)Z * es, st)) ||
         (e = palloc(&s->rt, (size_t)Z * es, st)) || (e = palloc(&s->r, R * es, st)) ||
         (e = palloc((void **)&s->grad, C * 4, st)) || (e = palloc((void **)&s->S, 8 * (size_t)M * g->desc.nv, st)) ||
@@ -1349,7 +1361,7 @@ extern "C" bsgd_status bsgd_state_create(const bsgd_geometry *g, const bsgd_solv
         (e = palloc((void **)&s->pair_upd, 8 * (size_t)M * N, st)) ||
         (s->st != BSGD_F32 && !p->image_plain && (e = palloc(&s->xlo, C * es, st))) ||
         (g->desc.nz > 1 && (e = palloc(&s->xT, C * es, st))) ||
-        (g->desc.nz > 1 && (e = palloc((void **)&s->gT, C * 4, st))) ||
+        (g->desc.nz > 1 && !s->w && (e = palloc((void **)&s->gT, C * 4, st))) ||
         (p->tv_lambda > 0 && (e = tv_work_alloc(g, s->tv))) ||
         (p->auto_mu && ((e = palloc((void **)&s->eud, 8 * (size_t)C, st)) ||
                         (e = palloc((void **)&s->eud_prev, 8 * (size_t)C, st)) ||
@@ -1368,6 +1380,7 @@ extern "C" bsgd_status bsgd_state_create(const bsgd_geometry *g, const bsgd_solv
         if (s->xlo) BSGD_CUDA(cudaMemsetAsync(s->xlo, 0, C * es, st));
         if (s->xT) BSGD_CUDA(cudaMemsetAsync(s->xT, 0, C * es, st));
         if (s->gT) BSGD_CUDA(cudaMemsetAsync(s->gT, 0, C * 4, st));
+        if (s->w) BSGD_CUDA(cudaMemsetAsync(s->w, 0, W * 4, st));   // the padding stays 0
         BSGD_CUDA(cudaMemsetAsync(s->d_iter, 0, 8, st));
         BSGD_CUDA(cudaMemsetAsync(s->ticket, 0, 8, st));
         BSGD_CUDA(cudaMemsetAsync(s->updates, 0, 8, st));
@@ -1452,6 +1465,7 @@ extern "C" bsgd_status bsgd_state_create(const bsgd_geometry *g, const bsgd_solv
     d.mu = s->d_mu;
     d.xT = s->xT;
     d.gT = s->gT;
+    d.w = s->w;
     d.eud = s->eud;
     *out = s;
     return BSGD_OK;
@@ -1469,7 +1483,7 @@ void state_release(bsgd_state *s, cudaStream_t st) {
         return;
     }
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
-    void *ptrs[] = {s->y, s->z, s->rt, s->r, s->xlo, s->xT, s->gT, s->grad, s->S, s->d_mu, s->work, s->cells,
+    void *ptrs[] = {s->y, s->z, s->rt, s->r, s->xlo, s->xT, s->gT, s->w, s->grad, s->S, s->d_mu, s->work, s->cells,
                     s->wband, s->d_iter, s->x0_flag, s->owned, s->wscratch, s->ticket, s->trace,
                     s->updates, s->pair_upd, s->eud, s->eud_prev, s->am_part, s->am};
     for (void *p : ptrs) pool_free(p, st);
@@ -1610,8 +1624,8 @@ size_t state_bytes(const bsgd_geometry_desc &d, int M, int N, const bsgd_solve_p
 // xT = transpose(x): the caller's image is the one to trust at the start of
 // every call (and after the TV prox rewrites it).
 static bsgd_status sync_xT(bsgd_state *s, void *x, cudaStream_t st) {
-    if (!s->xT) return BSGD_OK;
     const bsgd_geometry *g = s->g;
+    if (!s->xT) return BSGD_OK;
     const int tiles = ((g->desc.nx + 31) / 32) * ((g->desc.ny + 31) / 32) * g->desc.nz;
     const int gb = std::max(1, std::min(tiles, 152 * 8));
     if (s->st == BSGD_F32) transpose_kernel<float><<<gb, 256, 0, st>>>(g->dg, (const float *)x, (float *)s->xT);
@@ -1629,7 +1643,7 @@ static bsgd_status launch_update(bsgd_state *s, void *x, cudaStream_t st, bool d
     int64_t maxJ = 0;
     for (int j = 0; j < g->N; ++j) maxJ = std::max(maxJ, g->block_cols(j));
     // with the y-fastest copies: one CTA per 32 x 32 tile of the slab
-    const int64_t nt = s->gT ? ((g->desc.nx + 31) / 32) * (int64_t)((g->desc.ny + 31) / 32) *
+    const int64_t nt = s->xT ? ((g->desc.nx + 31) / 32) * (int64_t)((g->desc.ny + 31) / 32) *
                                    ((maxJ + (int64_t)g->desc.nx * g->desc.ny - 1) / ((int64_t)g->desc.nx * g->desc.ny))
                              : (maxJ + 1023) / 1024;
     // a grid of 4 CTAs per SM walks the tiles (the update is short: a second,
@@ -1664,6 +1678,13 @@ static bsgd_status launch_update(bsgd_state *s, void *x, cudaStream_t st, bool d
     return BSGD_OK;
 }
 
+// BP of the drawn pairs' residual change where no FP pass has done it.
+static bsgd_status state_bp(bsgd_state *s, int cols, cudaStream_t st) {
+    if (!s->w) return launch_bp_solve(s->g, s->dev, s->st, s->P, s->max_tiles, st);
+    BSGD_TRY(launch_column_change(s->g, s->dev, s->st, s->P, st));
+    return launch_column_solve(s->g, s->dev, cols, st);
+}
+
 // One iteration. `drawn`: its blocks were drawn by the previous iteration's
 // update launch; `draw_next`: this iteration's update launch also draws the
 // next iteration's blocks.
@@ -1687,14 +1708,18 @@ static bsgd_status one_iteration(bsgd_state *s, void *x, cudaStream_t st, bool d
     const bool replaying = s->replay && k >= s->replay_start && k < s->replay_start + s->replay_n;
     const bool fuse_multi = !s->fused && s->kN <= kMaxFusedCols &&
                             s->p.pair_sampling == BSGD_PAIRS_UNIFORM && !replaying;
+    const int cols = replaying ? std::min(s->P, g->N) : s->kN;   // distinct blocks, at most
     if (s->max_tiles > 0 && s->fused && !s->split) {
-        // one column block per iteration: FP, residual and BP in one pass
+        // one column block per iteration: FP, residual and BP in one pass (column
+        // form: the pass leaves the weights that the BP gathers)
         b = stage_begin(s, st);
         BSGD_TRY(launch_fpbp_solve(g, s->dev, x, s->st, s->P, s->max_tiles, st));
+        if (s->w) BSGD_TRY(launch_column_solve(g, s->dev, cols, st));
         stage_end(s, BSGD_STAGE_FPBP, b, 1, st);
     } else if (s->max_tiles > 0 && fuse_multi && !s->split) {
         b = stage_begin(s, st);
         BSGD_TRY(launch_fpbpm_solve(g, s->dev, x, s->st, s->kM, s->max_tiles_all, s->kN, st));
+        if (s->w) BSGD_TRY(launch_column_solve(g, s->dev, cols, st));
         stage_end(s, BSGD_STAGE_FPBP, b, 1, st);
     } else if (s->max_tiles > 0) {
         b = stage_begin(s, st);
@@ -1710,7 +1735,7 @@ static bsgd_status one_iteration(bsgd_state *s, void *x, cudaStream_t st, bool d
             stage_end(s, BSGD_STAGE_RESIDUAL, b, 1, st);
         }
         b = stage_begin(s, st);
-        BSGD_TRY(launch_bp_solve(g, s->dev, s->st, s->P, s->max_tiles, st));
+        BSGD_TRY(state_bp(s, cols, st));
         stage_end(s, BSGD_STAGE_BP, b, 1, st);
     }
     b = stage_begin(s, st);
@@ -1847,7 +1872,8 @@ extern "C" bsgd_status bsgd_shard_begin(bsgd_state *s, void *x, float *exchange,
     fill_sample_args(s, A, k);
     sample_kernel<<<1, kSampleThreads, 0, st>>>(A);
     BSGD_CUDA(cudaGetLastError());
-    if (s->max_tiles > 0) BSGD_TRY(launch_fp_solve(g, s->dev, x, s->st, s->P, s->max_tiles, false, st));
+    if (s->max_tiles > 0)
+        BSGD_TRY(launch_fp_solve(g, s->dev, x, s->st, s->P, s->max_tiles, false, st));
     dim3 grid((g->desc.nv + kResRows - 1) / kResRows, g->max_views, s->kM);
     if (s->st == BSGD_F32) shard_partial_kernel<float><<<grid, 256, 0, st>>>(g->dg, s->dev, exchange);
     else if (s->st == BSGD_BF16) shard_partial_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->dg, s->dev, exchange);
@@ -1866,7 +1892,7 @@ extern "C" bsgd_status bsgd_shard_end(bsgd_state *s, void *x, const float *excha
     else if (s->st == BSGD_BF16) shard_residual_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->dg, s->dev, exchange);
     else shard_residual_kernel<__half><<<grid, 256, 0, st>>>(g->dg, s->dev, exchange);
     BSGD_CUDA(cudaGetLastError());
-    if (s->max_tiles > 0) BSGD_TRY(launch_bp_solve(g, s->dev, s->st, s->P, s->max_tiles, st));
+    if (s->max_tiles > 0) BSGD_TRY(state_bp(s, s->kN, st));
     BSGD_TRY(launch_update(s, x, st, false));
     s->iters += 1;
     return BSGD_OK;
@@ -1949,6 +1975,8 @@ struct CkptPart {
     void *dev;
     size_t bytes;
 };
+
+constexpr size_t kCkptTracePart = 9;   // the trace is the ninth part
 
 // The device arrays of a checkpoint, in blob order; trace rows = iterations
 // recorded so far.
@@ -2042,17 +2070,35 @@ extern "C" bsgd_status bsgd_state_restore(bsgd_state *s, const void *host, int64
     const std::vector<CkptPart> parts = ckpt_parts(s, h.trace_rows);
     size_t need = 0;
     for (const CkptPart &q : parts) need += q.bytes;
+    // a state that scattered kept part of g y-fastest, after the trace
+    const size_t C = (size_t)s->g->n_cols();
+    const bool old_gT = s->w && (int64_t)(need + C * 4) == h.payload;
+    if (old_gT) need += C * 4;
     if ((int64_t)need != h.payload || bytes < (int64_t)sizeof(CkptHeader) + h.payload)
         return fail(BSGD_ERR_INVALID_ARG, "checkpoint truncated");
     cudaStream_t st = (cudaStream_t)stream;
     if (h.pair_sampling != s->p.pair_sampling || h.cells != s->p.cells || h.n_cells != s->n_cells)
         BSGD_TRY(bsgd_state_set_sampling(s, h.pair_sampling, h.cells, h.n_cells, stream));
-    const char *in = static_cast<const char *>(host) + sizeof h;
-    for (const CkptPart &q : parts) {
-        if (q.bytes) BSGD_CUDA(cudaMemcpyAsync(q.dev, in, q.bytes, cudaMemcpyHostToDevice, st));
-        in += q.bytes;
-    }
-    BSGD_CUDA(cudaStreamSynchronize(st));
+    float *gT = nullptr;
+    if (old_gT) BSGD_TRY(palloc((void **)&gT, C * 4, st));
+    auto load = [&]() -> bsgd_status {
+        const char *in = static_cast<const char *>(host) + sizeof h;
+        for (size_t k = 0; k < parts.size(); ++k) {
+            const CkptPart &q = parts[k];
+            if (q.bytes) BSGD_CUDA(cudaMemcpyAsync(q.dev, in, q.bytes, cudaMemcpyHostToDevice, st));
+            in += q.bytes;
+            if (gT && k + 1 == kCkptTracePart) {
+                BSGD_CUDA(cudaMemcpyAsync(gT, in, C * 4, cudaMemcpyHostToDevice, st));
+                BSGD_TRY(plain_add_transposed(s->g, gT, s->grad, 0, s->g->N, st));
+                in += C * 4;
+            }
+        }
+        BSGD_CUDA(cudaStreamSynchronize(st));
+        return BSGD_OK;
+    };
+    const bsgd_status le = load();
+    pool_free(gT, st);
+    BSGD_TRY(le);
     s->iters = h.iters;
     cudaFree(s->replay);   // a replay in progress belongs to the state that was replaced
     s->replay = nullptr;

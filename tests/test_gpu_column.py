@@ -3,7 +3,8 @@ oracle, at the sizes where its pieces end: planes past a whole chunk of 32, an
 odd nz (the source's height inside a voxel), a level detector row, slabs on both
 sides of the source's height, detectors finer than half a voxel (more than one
 pair of rows per crossing) and coarser than one, columns past a CTA's tile,
-rays along the axes, 16-bit residuals."""
+rays along the axes, 16-bit residuals, and the solver's form of it (several
+column blocks, drawn detector cells)."""
 import numpy as np
 import pytest
 
@@ -12,6 +13,7 @@ from helpers import gpu_geom, oracle_geom, rel_l2
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+from oracle import bsgd as OB  # noqa: E402
 from oracle import projector as P  # noqa: E402
 from paper_1903_11874_gb300 import binding as B  # noqa: E402
 from paper_1903_11874_gb300 import synth  # noqa: E402
@@ -115,3 +117,35 @@ def test_infinite_and_nan_weights_stay_on_their_rays():
     assert np.all(np.isnan(got[a > 1e-3]))
     assert np.all(np.isposinf(got[(b > 1e-3) & ~near_a]))
     assert np.all(got[~near_a & ~near_b] == 0.0)
+
+
+@pytest.mark.parametrize("kN,cells,storage", [(1, "none", "f32"), (2, "none", "f32"), (2, "geometric", "f32"),
+                                              (2, "uniform", "f32"), (2, "none", "bf16")])
+def test_solver(kN, cells, storage):
+    """BSGD at the smallest size whose solver gathers, against the oracle with the
+    same draws; odd nv (a level row) and uneven slabs."""
+    M = 1 if kN == 1 else 2
+    s = cone(128, 126, 66 if kN == 1 else 64, 50, 80, 71, 3.2, M=M, N=2, dso=300.0, dsd=600.0)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    xt = synth.ellipsoid_phantom(128, 126, s["nz"], 4, seed=1).reshape(-1).astype(np.float64) * 0.01
+    y = P.fp(og, xt).reshape(-1).astype(np.float32)
+    mu, iters = 2e-5, 4
+    kinds = {"none": B.CELLS_NONE, "geometric": B.CELLS_GEOMETRIC, "uniform": B.CELLS_UNIFORM}
+    n_cells = 1 if cells == "none" else 4
+    prm = B.SolveParams(alpha=1 / M, gamma=kN / 2, step_rule=B.STEP_FIXED, mu=mu, seed=5, cells=kinds[cells],
+                        n_cells=n_cells, storage=B.F32 if storage == "f32" else B.BF16)
+    st = B.State(gg, prm, torch.from_numpy(y).to(DEV))
+    x = torch.zeros(og.n_cols, device=DEV, dtype=torch.float32 if storage == "f32" else torch.bfloat16)
+    st.block_step(x, iters)
+    po = OB.Params(M, 2, 1 / M, kN / 2, mu, seed=5, cells=cells, n_cells=n_cells)
+    ost = OB.bsgd(og, y.astype(np.float64), po, iters)
+    assert rel_l2(x.cpu().double().numpy(), ost.x) <= (1e-5 if storage == "f32" else 1e-2)
+    q = st.query()
+    assert abs(q["residual_norm"] - ost.residual_norm()) <= (1e-5 if storage == "f32" else 1e-2) * ost.residual_norm()
+    # a checkpoint carries the gathered gradient
+    blob, x1 = st.save(), x.clone()
+    st.block_step(x, 2)
+    st2 = B.State(gg, prm, torch.from_numpy(y).to(DEV))
+    st2.restore(blob)
+    st2.block_step(x1, 2)
+    assert torch.equal(x, x1)
