@@ -174,23 +174,30 @@ __global__ void __launch_bounds__(256) column_change_kernel(const DeviceGeom G, 
 
 }  // namespace
 
+// Lanes that the gather spends per ray that meets a voxel of its column: chunks
+// of 32 planes that `planes` do not fill, and rows further apart than a voxel,
+// cost as much as full ones, while the scatter follows the rays there are.
+static double gather_waste(const bsgd_geometry *g, int planes) {
+    const bsgd_geometry_desc &d = g->desc;
+    return (planes + 31) / 32 * 32.0 / planes * (d.dv * d.dso / d.dsd / d.dz);
+}
+
 // Whether the back projection of `views` views into `planes` planes gathers. A
 // warp runs through all views of its column (0.43 us each, whatever the other
 // warps do), so small slabs seen from many views scatter instead: 64 x 64 x 32
 // from 360 views 151 us scattered, 164 gathered; 64^3 from 90 views 114 and 66
 // us; 48 x 48 x 32 from 24 views 35 and 23 us; 32^3 from 90 views 35 and 39 us.
+// Full chunks gather 2.1 times as fast as they scatter at a waste of 0.8, 1.2
+// times at 1.4.
 bool column_bp_pays(const bsgd_geometry *g, int planes, int views) {
     const int64_t voxels = (int64_t)g->desc.nx * g->desc.ny * planes;
-    return g->dg.cray && voxels >= (views <= 32 ? 64000 : 160000);
+    return g->dg.cray && planes > 0 && voxels >= (views <= 32 ? 64000 : 160000) && gather_waste(g, planes) <= 1.7;
 }
 
 bsgd_status column_tables(bsgd_geometry *g) {
     const bsgd_geometry_desc &d = g->desc;
     DeviceGeom &dg = g->dg;
     if (d.kind != BSGD_CONE3D || d.nz < 2 || d.nv < 2) return BSGD_OK;
-    // rows more than two voxels apart at the axis: most voxels of a column meet
-    // no ray of a view, and the ray-driven scatter has less to do
-    if (d.dv * d.dso / d.dsd > 2.0 * d.dz) return BSGD_OK;
     // rows are found by an addition that holds them in 22 bits
     const double near = d.dso - 0.5 * std::hypot(d.nx * d.dx, d.ny * d.dy);
     if (d.nv > (1 << 20) || d.dz * d.dsd / (near * d.dv) > 1e3) return BSGD_OK;
@@ -255,14 +262,17 @@ bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const
 // 256^2 x 32 from 45 views 432 / 390, 192^2 x 32 from 22 160 / 148, 96^2 x 32
 // from 45 83 / 81, 256^2 x 32 from 11 162 / 169, 256^2 x 16 from 45 258 / 312;
 // two blocks: 256^2 x 32 from 45 887 / 758, 128^2 x 32 from 11 120 / 90, 96^2 x
-// 12 from 22 70 / 68.
+// 12 from 22 70 / 68. At a waste of 1.58 (205 x 170 x 40 from 59 views, rows a
+// voxel apart) 284 / 333.
 // With detector cells one block's pass traces a fraction of the rays that the
 // gather lists: 160^2 x 32 from 45 views 90 / 109, 256^2 x 32 258 / 260.
 size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells) {
     if (!g->dg.cray || (cells && kN == 1)) return 0;
     const int planes = g->desc.nz / g->N;   // of the thinnest slab
     const int64_t work = (int64_t)g->desc.nx * g->desc.ny * planes * kN * g->max_views * kM;
-    if (planes < 28 || work < (kN > 1 ? 10000000 : 25000000)) return 0;
+    if (planes < 28 || work < (kN > 1 ? 10000000 : 25000000) ||
+        gather_waste(g, (g->desc.nz + g->N - 1) / g->N) > 1.12)
+        return 0;
     return column_weights_len(g, kM * kN);
 }
 

@@ -31,10 +31,10 @@ CASES = {
     "odd_height_level_row": cone(67, 64, 65, 8, 81, 91, 1.9),
     "level_row_in_a_face": cone(64, 64, 64, 8, 80, 81, 2.1),
     "fine_rows": cone(64, 64, 40, 4, 200, 150, 0.7),
-    "coarse_rows": cone(70, 66, 64, 16, 40, 40, 3.9),
-    "nine_chunks": cone(40, 40, 260, 4, 50, 120, 3.4),
+    "coarse_rows": cone(70, 66, 64, 16, 50, 48, 3.2),
+    "nine_chunks": cone(40, 40, 260, 4, 50, 130, 2.8),
     "short_distance": cone(64, 64, 48, 8, 96, 64, 1.6, dso=80.0, dsd=200.0),
-    "rise_of_most_of_a_voxel": cone(48, 48, 72, 8, 60, 60, 3.2, dso=72.0, dsd=144.0),
+    "rise_of_most_of_a_voxel": cone(48, 48, 64, 8, 84, 84, 2.2, dso=72.0, dsd=144.0),
 }
 
 
@@ -125,7 +125,7 @@ def test_solver(kN, cells, storage):
     """BSGD at the smallest size whose solver gathers, against the oracle with the
     same draws; odd nv (a level row) and uneven slabs."""
     M = 1 if kN == 1 else 2
-    s = cone(128, 126, 66 if kN == 1 else 64, 50, 80, 71, 3.2, M=M, N=2, dso=300.0, dsd=600.0)
+    s = cone(128, 126, 63 if kN == 1 else 64, 52, 110, 71, 2.2, M=M, N=2, dso=300.0, dsd=600.0)
     og, gg = oracle_geom(s), gpu_geom(s)
     xt = synth.ellipsoid_phantom(128, 126, s["nz"], 4, seed=1).reshape(-1).astype(np.float64) * 0.01
     y = P.fp(og, xt).reshape(-1).astype(np.float32)
