@@ -61,6 +61,7 @@ __device__ inline int pick_weighted(double u, const double *w, int n, int stride
 constexpr int kSampleThreads = 256;
 constexpr int kMaxSampleBlocks = 1024;
 constexpr int kMaxResidualPairs = 1024;
+constexpr int kDrawLists = 16;         // iterations whose draws a state holds
 constexpr int kSampleSmemS = 2048;     // residual-table entries staged in shared memory
 
 // One iteration's draw (Algorithm 1's selection step; Algorithm 2's per-view
@@ -325,10 +326,23 @@ __device__ void sample_body(const SampleArgs &A, const double *pre_w = nullptr) 
         for (int q = 1 + 2 * np + np * G.max_views + tid; q < A.stride; q += blockDim.x) t[q] = -1;
     }
     __syncthreads();
-    if (tid == 0) *A.iter = it + 1;
+    if (tid == 0 && A.iter) *A.iter = it + 1;
 }
 
 __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs A) { sample_body(A); }
+
+// The draws of iterations A.it .. A.it + gridDim.x - 1, which do not depend on
+// the residual: a CTA each, into the lists that their iterations read. One draw
+// is a chain of memory latencies (9.4 us as a launch, and as part of an update
+// that it outlasts on small images); kDrawLists of them take no longer.
+__global__ void __launch_bounds__(kSampleThreads) sample_ahead_kernel(SampleArgs A, Work *lists, int *cells) {
+    const int64_t it = A.it + blockIdx.x;
+    A.it = it;
+    A.work = lists + it % kDrawLists;
+    A.cells = cells + it % kDrawLists * (int64_t)kMaxPairs * A.G.max_views;
+    if (blockIdx.x + 1 < gridDim.x) A.iter = nullptr;   // the last one advances the counter
+    sample_body(A);
+}
 
 // pair_upd[i][j] = voxel-ray updates of every whole view of row block i in
 // column block j (the cell counts summed).
@@ -1350,8 +1364,8 @@ bsgd_status bsgd::state_create(const bsgd_geometry *g, const bsgd_solve_params *
     if ((e = palloc(&s->y, R * es, st)) || (e = palloc(&s->z, (size_t)Z * es, st)) ||
         (e = palloc(&s->rt, (size_t)Z * es, st)) || (e = palloc(&s->r, R * es, st)) ||
         (e = palloc((void **)&s->grad, C * 4, st)) || (e = palloc((void **)&s->S, 8 * (size_t)M * g->desc.nv, st)) ||
-        (e = palloc((void **)&s->d_mu, 8, st)) || (e = palloc((void **)&s->work, 2 * sizeof(Work), st)) ||
-        (e = palloc((void **)&s->cells, 2 * 4 * (size_t)kMaxPairs * g->max_views, st)) ||
+        (e = palloc((void **)&s->d_mu, 8, st)) || (e = palloc((void **)&s->work, kDrawLists * sizeof(Work), st)) ||
+        (e = palloc((void **)&s->cells, kDrawLists * 4 * (size_t)kMaxPairs * g->max_views, st)) ||
         (e = palloc((void **)&s->wband, 4 * g->wband.size(), st)) ||
         (e = palloc((void **)&s->d_iter, 8, st)) || (e = palloc((void **)&s->x0_flag, 8, st)) ||
         (e = palloc((void **)&s->wscratch, 8 * (size_t)kMaxResidualPairs, st)) ||
@@ -1384,8 +1398,8 @@ bsgd_status bsgd::state_create(const bsgd_geometry *g, const bsgd_solve_params *
         BSGD_CUDA(cudaMemsetAsync(s->d_iter, 0, 8, st));
         BSGD_CUDA(cudaMemsetAsync(s->ticket, 0, 8, st));
         BSGD_CUDA(cudaMemsetAsync(s->updates, 0, 8, st));
-        BSGD_CUDA(cudaMemsetAsync(s->work, 0, 2 * sizeof(Work), st));
-        BSGD_CUDA(cudaMemsetAsync(s->cells, 0xff, 2 * 4 * (size_t)kMaxPairs * g->max_views, st));
+        BSGD_CUDA(cudaMemsetAsync(s->work, 0, kDrawLists * sizeof(Work), st));
+        BSGD_CUDA(cudaMemsetAsync(s->cells, 0xff, kDrawLists * 4 * (size_t)kMaxPairs * g->max_views, st));
         BSGD_CUDA(cudaMemcpyAsync(s->wband, g->wband.data(), 4 * g->wband.size(),
                                   cudaMemcpyHostToDevice, st));
         BSGD_TRY(norm_table(g, s->r, s->st, s->S, st));
@@ -1498,12 +1512,11 @@ extern "C" bsgd_status bsgd_state_destroy(bsgd_state *s) {
     return BSGD_OK;
 }
 
-// The work list and the chosen cells are double-buffered by iteration parity,
-// so the draw of iteration k + 1 can run while iteration k's update reads its
-// own list.
-static Work *work_buf(const bsgd_state *s, int64_t k) { return s->work + (k & 1); }
+// The work list and the chosen cells of iteration k are buffer k % kDrawLists, so
+// that later iterations can be drawn while k's update reads its own list.
+static Work *work_buf(const bsgd_state *s, int64_t k) { return s->work + k % kDrawLists; }
 static int *cells_buf(const bsgd_state *s, int64_t k) {
-    return s->cells + (k & 1) * (size_t)kMaxPairs * s->g->max_views;
+    return s->cells + k % kDrawLists * (size_t)kMaxPairs * s->g->max_views;
 }
 
 static void fill_sample_args(const bsgd_state *s, SampleArgs &A, int64_t k) {
@@ -1605,7 +1618,7 @@ size_t state_bytes(const bsgd_geometry_desc &d, int M, int N, const bsgd_solve_p
     if (es != 4 && !p.image_plain) b += C * es;        // low-order image term
     if (d.nz > 1) b += C * (es + 4);                   // y-fastest copies of x and g
     b += 8 * (size_t)M * d.nv;                         // residual table
-    b += 4 * (size_t)kMaxPairs * maxV + 8 * (size_t)M * N + sizeof(Work) + 64;
+    b += kDrawLists * (4 * (size_t)kMaxPairs * maxV + sizeof(Work)) + 8 * (size_t)M * N + 64;
     b += 4 * (size_t)65536 * stride;                   // trace
     b += 8 * (size_t)N * d.n_views * cells * (p.cells == BSGD_CELLS_GEOMETRIC ? 2 : 1);
     // geometry tables
@@ -1685,10 +1698,10 @@ static bsgd_status state_bp(bsgd_state *s, int cols, cudaStream_t st) {
     return launch_column_solve(s->g, s->dev, cols, st);
 }
 
-// One iteration. `drawn`: its blocks were drawn by the previous iteration's
-// update launch; `draw_next`: this iteration's update launch also draws the
-// next iteration's blocks.
-static bsgd_status one_iteration(bsgd_state *s, void *x, cudaStream_t st, bool drawn,
+// One iteration. `drawn`: its blocks are drawn already; otherwise `ahead` (at
+// least 1) iterations are drawn at once. `draw_next`: this iteration's update
+// launch also draws the next iteration's blocks.
+static bsgd_status one_iteration(bsgd_state *s, void *x, cudaStream_t st, bool drawn, int ahead,
                                  bool draw_next) {
     const bsgd_geometry *g = s->g;
     const int64_t k = s->iters;
@@ -1699,7 +1712,7 @@ static bsgd_status one_iteration(bsgd_state *s, void *x, cudaStream_t st, bool d
         SampleArgs A;
         fill_sample_args(s, A, k);
         b = stage_begin(s, st);
-        sample_kernel<<<1, kSampleThreads, 0, st>>>(A);
+        sample_ahead_kernel<<<ahead, kSampleThreads, 0, st>>>(A, s->work, s->cells);
         BSGD_CUDA(cudaGetLastError());
         stage_end(s, BSGD_STAGE_SAMPLE, b, 1, st);
     }
@@ -1787,7 +1800,15 @@ extern "C" bsgd_status bsgd_block_step(bsgd_state *s, void *x, int n_iters, void
     if (s->owned) return fail(BSGD_ERR_STATE, "a sharded state steps through bsgd_shard_begin / _end");
     if (n_iters > 0) BSGD_TRY(sync_xT(s, x, st));
     if (n_iters > 0 && s->iters == 0 && !s->zero_start) BSGD_TRY(warm_start(s, x, st));
-    for (int k = 0; k < n_iters; ++k) BSGD_TRY(one_iteration(s, x, st, k > 0, k + 1 < n_iters));
+    // uniform pairs (and their cells) do not depend on the residual: drawn
+    // kDrawLists iterations at a time; residual-weighted pairs one iteration
+    // ahead, beside the update
+    const bool ahead = s->p.pair_sampling == BSGD_PAIRS_UNIFORM;
+    for (int k = 0; k < n_iters; ++k) {
+        const bool drawn = ahead ? k % kDrawLists != 0 : k > 0;
+        BSGD_TRY(one_iteration(s, x, st, drawn, ahead ? std::min(kDrawLists, n_iters - k) : 1,
+                               !ahead && k + 1 < n_iters));
+    }
     return BSGD_OK;
 }
 
