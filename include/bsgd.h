@@ -158,8 +158,9 @@ bsgd_status bsgd_forward_project(const bsgd_geometry *g, const void *x, bsgd_dty
  *  x: device, batch * n_cols float32 (BSGD_F32 only: the sums are kept in
  *     float). With accumulate = 0 the voxels of the selected
  *     column blocks are cleared first; other voxels are untouched.
- * Larger cone-beam volumes gather (the same sum in every run) from weights that
- * the call lays out in the library's memory pool: n_views of the row blocks (at
+ * 2D images of 4096 pixels or more gather (the same sum in every run). Larger
+ * cone-beam volumes do so too, from weights that the call lays out in the
+ * library's memory pool: n_views of the row blocks (at
  * most 64 blocks at a time) * nu * (nv and some padding) floats. Otherwise, or
  * if the pool has no room, the rays scatter: not bit-reproducible run to run
  * (atomic order), results agree to float rounding; the views whose rays run

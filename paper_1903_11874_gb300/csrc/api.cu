@@ -144,6 +144,10 @@ extern "C" bsgd_status bsgd_back_project(const bsgd_geometry *g, const void *r, 
                 const int64_t v0 = (int64_t)g->plane_start[run.first] * g->dg.plane_stride;
                 const int64_t v1 = (int64_t)g->plane_start[run.second] * g->dg.plane_stride;
                 PlainLaunch L{rows.data(), (int)rows.size(), run.first, run.second, 0};
+                if (slice_bp_pays(g, g->plane_start[run.second] - g->plane_start[run.first], views)) {
+                    BSGD_TRY(launch_bp_slice(g, L, rb, rt, xb, scale, accumulate, st));
+                    continue;
+                }
                 if (w && gathers(run)) {
                     BSGD_TRY(launch_bp_column(g, L, rb, rt, xb, scale, accumulate, w, st));
                     continue;

@@ -53,7 +53,7 @@ struct ViewRay {
 };
 static_assert(sizeof(ViewRay) == 64, "ViewRay is 4 x float4");
 
-// Line of one (view, detector column) of a cone beam in the xy plane: offsets
+// Line of one (view, detector column) in the xy plane: offsets
 // from the volume's centre where the ray parameter equals the rotation axis's
 // (high and low part), 1 / slope and slope per axis (column.cuh).
 struct ColRay {
@@ -87,8 +87,14 @@ struct DeviceGeom {
     int M, N, axis, max_views;
     int64_t n_rows, n_cols;
     int plane_stride;          // voxels per plane along the block axis
-    // Column form of a cone beam (column.cuh); cray is null where it is not used
+    // Column form of a cone beam (column.cuh), nvp = 0 where it is not used; lines
+    // of a 2D kind
     const ColRay *cray;        // n_views x nu
+    // 2D kinds (else null): the same line as arrays of n_views x nu, so that the
+    // lanes of neighbouring columns read neighbouring addresses
+    const float2 *sx, *sy;     // {xh, xl}, {yh, yl}
+    const float2 *si;          // {ix, iy}
+    const float *slen;         // length of the ray (mm)
     float tc;                  // ray parameter of the rotation axis
     float zs;                  // source height (voxels from the volume's low face)
     float vstep;               // z slope per detector row
@@ -125,6 +131,7 @@ struct bsgd_geometry {
     unsigned char *d_view_yfast = nullptr;
     int64_t *d_zoff = nullptr;
     bsgd::ColRay *d_cray = nullptr;
+    float2 *d_slice = nullptr;
     bsgd::DeviceGeom dg{};
     // Filled on first use by a solver state and kept for the geometry's life
     // (index: number of detector cells 1, 2 or 4): exact voxel-ray update
@@ -202,6 +209,10 @@ bsgd_status launch_count(const bsgd_geometry *g, const PlainLaunch &L,
 bsgd_status column_tables(bsgd_geometry *g);
 bool column_bp_pays(const bsgd_geometry *g, int planes, int views);
 size_t column_weights_len(const bsgd_geometry *g, int n_rb);
+// The same for images of a 2D kind: a thread per pixel, no weights.
+bool slice_bp_pays(const bsgd_geometry *g, int rows, int views);
+bsgd_status launch_bp_slice(const bsgd_geometry *g, const PlainLaunch &L, const void *r, bsgd_dtype rt,
+                            float *x, float scale, int accumulate, cudaStream_t st);
 size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells);
 bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const void *r,
                              bsgd_dtype rt, float *x, float scale, int accumulate, float *w,

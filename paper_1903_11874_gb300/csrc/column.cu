@@ -11,15 +11,16 @@ namespace {
 
 // Lines of every (view, detector column), from the FP32 ray table (the same rays
 // as the incremental walk's), in FP64.
-__global__ void column_tables_kernel(const DeviceGeom G, ColRay *__restrict__ cray) {
+__global__ void column_tables_kernel(const DeviceGeom G, ColRay *__restrict__ cray, float2 *__restrict__ slice) {
     const int64_t n = (int64_t)G.n_views * G.nu;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x) {
         const ViewRay &R = G.rays[k / G.nu];
         const float fu = (float)(int)(k % G.nu) - 0.5f * (float)(G.nu - 1);
-        const float dx = fmaf(fu, R.cu[0], R.c0[0]) - R.p0[0], dy = fmaf(fu, R.cu[1], R.c0[1]) - R.p0[1];
-        const double X = (double)R.p0[0] + (double)G.tc * dx - 0.5 * G.nx;
-        const double Y = (double)R.p0[1] + (double)G.tc * dy - 0.5 * G.ny;
+        const float x0 = fmaf(fu, R.pu[0], R.p0[0]), y0 = fmaf(fu, R.pu[1], R.p0[1]);
+        const float dx = fmaf(fu, R.cu[0], R.c0[0]) - x0, dy = fmaf(fu, R.cu[1], R.c0[1]) - y0;
+        const double X = (double)x0 + (double)G.tc * dx - 0.5 * G.nx;
+        const double Y = (double)y0 + (double)G.tc * dy - 0.5 * G.ny;
         ColRay c;
         c.xh = (float)X;
         c.yh = (float)Y;
@@ -32,7 +33,13 @@ __global__ void column_tables_kernel(const DeviceGeom G, ColRay *__restrict__ cr
         // a line lying in a face belongs to the cell on its + side
         if (dx == 0.f) c.xl += 1e-9f;
         if (dy == 0.f) c.yl += 1e-9f;
-        cray[k] = c;
+        if (cray) cray[k] = c;
+        if (slice) {
+            slice[k] = make_float2(c.xh, c.xl);
+            slice[n + k] = make_float2(c.yh, c.yl);
+            slice[2 * n + k] = make_float2(c.ix, c.iy);
+            reinterpret_cast<float *>(slice + 3 * n)[k] = sqrtf(column_length2(G, c));
+        }
     }
 }
 
@@ -172,6 +179,48 @@ __global__ void __launch_bounds__(256) column_change_kernel(const DeviceGeom G, 
     }
 }
 
+// Back projection of a 2D kind into rows [y0, y1) of the image, as a gather: a
+// CTA takes 32 pixels of a row, its 8 warps every 8th view each; a thread tests
+// the detector columns whose shadow its pixel is in (one to three) and adds
+// weight x chord. 256^2 pixels from 360 fan views of 384 bins (30 M updates): 193
+// us as a scatter, whose atomics meet on 65536 addresses, 136 us gathered (168 us
+// with the lines as 32-byte records: a warp's load then spans ten 128-byte
+// lines). What bounds it: issue slots, half of them for finding the columns, and
+// lanes that wait for the ones with three columns.
+template <bool kParallel, typename T>
+__global__ void __launch_bounds__(256) bp_slice_kernel(const DeviceGeom G, const RowSel R, int y0,
+                                                       const T *__restrict__ r, float scale,
+                                                       float *__restrict__ x, int add) {
+    __shared__ float s[8][32];
+    const int tiles = (G.nx + 31) / 32, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int xx = (int)(blockIdx.x % tiles) * 32 + lane, y = y0 + (int)(blockIdx.x / tiles);
+    const float fx = (float)xx - 0.5f * (float)G.nx, fy = (float)y - 0.5f * (float)G.ny;
+    float acc = 0.f;
+    for (int k = 0; k < R.n; ++k) {
+        const int *views = G.block_views + R.ids[k] * G.max_views;
+        const int n = G.block_nviews[R.ids[k]];
+        for (int q = warp; q < n; q += 8) {
+            const int a = views[q];
+            const int2 ur = cell_columns<kParallel>(G, a, (float)xx + 0.5f, (float)y + 0.5f);
+            for (int u = ur.x; u <= ur.y; ++u) {
+                const int i = a * G.nu + u;
+                const float2 X = __ldg(G.sx + i), Y = __ldg(G.sy + i), I = __ldg(G.si + i);
+                const float wl = ldf(r + i) * scale * __ldg(G.slen + i);
+                float t0, t1;
+                cell_interval(ColRay{X.x, X.y, I.x, 0.f, Y.x, Y.y, I.y, 0.f}, fx, fy, t0, t1);
+                if (t1 > t0) acc = fmaf(t1 - t0, wl, acc);
+            }
+        }
+    }
+    s[warp][lane] = acc;
+    __syncthreads();
+    if (warp > 0 || xx >= G.nx) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) acc += s[q][lane];
+    float *p = x + (int64_t)y * G.nx + xx;
+    *p = add ? *p + acc : acc;
+}
+
 }  // namespace
 
 // Lanes that the gather spends per ray that meets a voxel of its column: chunks
@@ -191,13 +240,36 @@ static double gather_waste(const bsgd_geometry *g, int planes) {
 // times at 1.4.
 bool column_bp_pays(const bsgd_geometry *g, int planes, int views) {
     const int64_t voxels = (int64_t)g->desc.nx * g->desc.ny * planes;
-    return g->dg.cray && planes > 0 && voxels >= (views <= 32 ? 64000 : 160000) && gather_waste(g, planes) <= 1.7;
+    return g->dg.nvp > 0 && planes > 0 && voxels >= (views <= 32 ? 64000 : 160000) && gather_waste(g, planes) <= 1.7;
+}
+
+static bsgd_status fill_tables(bsgd_geometry *g, bool slice) {
+    DeviceGeom &dg = g->dg;
+    const int64_t n = (int64_t)g->desc.n_views * g->desc.nu;
+    if (slice) BSGD_CUDA(cudaMalloc((void **)&g->d_slice, 28 * (size_t)n));
+    else BSGD_CUDA(cudaMalloc((void **)&g->d_cray, sizeof(ColRay) * (size_t)n));
+    const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 152 * 16));
+    column_tables_kernel<<<gb, 128>>>(dg, g->d_cray, g->d_slice);
+    BSGD_CUDA(cudaGetLastError());
+    BSGD_CUDA(cudaStreamSynchronize(0));
+    dg.cray = g->d_cray;
+    if (slice) {
+        dg.sx = g->d_slice;
+        dg.sy = g->d_slice + n;
+        dg.si = g->d_slice + 2 * n;
+        dg.slen = reinterpret_cast<float *>(g->d_slice + 3 * n);
+    }
+    return BSGD_OK;
 }
 
 bsgd_status column_tables(bsgd_geometry *g) {
     const bsgd_geometry_desc &d = g->desc;
     DeviceGeom &dg = g->dg;
-    if (d.kind != BSGD_CONE3D || d.nz < 2 || d.nv < 2) return BSGD_OK;
+    if (d.kind != BSGD_CONE3D) {
+        dg.tc = d.kind == BSGD_PAR2D ? 0.5f : (float)(d.dso / d.dsd);
+        return fill_tables(g, true);
+    }
+    if (d.nz < 2 || d.nv < 2) return BSGD_OK;
     // rows are found by an addition that holds them in 22 bits
     const double near = d.dso - 0.5 * std::hypot(d.nx * d.dx, d.ny * d.dy);
     if (d.nv > (1 << 20) || d.dz * d.dsd / (near * d.dv) > 1e3) return BSGD_OK;
@@ -214,14 +286,7 @@ bsgd_status column_tables(bsgd_geometry *g) {
     dg.vslack = (float)(32.0 * change * 1.01);
     dg.vpad = (int)std::ceil(33.0 * rows + (2.0 * d.nz + 32.0) * change) + 8;
     dg.nvp = (d.nv + 2 * dg.vpad + 7) / 8 * 8;
-    BSGD_CUDA(cudaMalloc((void **)&g->d_cray, sizeof(ColRay) * (size_t)d.n_views * d.nu));
-    const int64_t n = (int64_t)d.n_views * d.nu;
-    const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 152 * 16));
-    column_tables_kernel<<<gb, 128>>>(dg, g->d_cray);
-    BSGD_CUDA(cudaGetLastError());
-    BSGD_CUDA(cudaStreamSynchronize(0));
-    dg.cray = g->d_cray;
-    return BSGD_OK;
+    return fill_tables(g, false);
 }
 
 size_t column_weights_len(const bsgd_geometry *g, int n_rb) {
@@ -267,13 +332,43 @@ bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const
 // With detector cells one block's pass traces a fraction of the rays that the
 // gather lists: 160^2 x 32 from 45 views 90 / 109, 256^2 x 32 258 / 260.
 size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells) {
-    if (!g->dg.cray || (cells && kN == 1)) return 0;
+    if (g->dg.nvp == 0 || (cells && kN == 1)) return 0;
     const int planes = g->desc.nz / g->N;   // of the thinnest slab
     const int64_t work = (int64_t)g->desc.nx * g->desc.ny * planes * kN * g->max_views * kM;
     if (planes < 28 || work < (kN > 1 ? 10000000 : 25000000) ||
         gather_waste(g, (g->desc.nz + g->N - 1) / g->N) > 1.12)
         return 0;
     return column_weights_len(g, kM * kN);
+}
+
+// Whether the back projection of a 2D kind into `rows` image rows gathers: us
+// scattered / gathered, 64^2 from 90 views 15.4 / 14.4, 128^2 from 60 17.4 /
+// 10.5, 100 x 17 of a strip from 180 20.1 / 20.1, 512^2 from 720 930 / 865.
+// Below 4096 pixels the two are level.
+bool slice_bp_pays(const bsgd_geometry *g, int rows, int views) {
+    return g->dg.sx && (int64_t)g->desc.nx * rows >= 4096 && views >= 1;
+}
+
+bsgd_status launch_bp_slice(const bsgd_geometry *g, const PlainLaunch &L, const void *r, bsgd_dtype rt,
+                            float *x, float scale, int accumulate, cudaStream_t st) {
+    const int y0 = g->plane_start[L.j0], y1 = g->plane_start[L.j1];
+    const unsigned grid = (unsigned)((g->desc.nx + 31) / 32) * (y1 - y0);
+    for (int k = 0; k < L.n_rb; k += 64) {
+        RowSel R{};
+        R.n = std::min(64, L.n_rb - k);
+        for (int t = 0; t < R.n; ++t) R.ids[t] = L.row_ids[k + t];
+        const int add = accumulate || k > 0;
+#define SLICE_GO(T)                                                                                            \
+    if (g->desc.kind == BSGD_PAR2D)                                                                            \
+        bp_slice_kernel<true, T><<<grid, 256, 0, st>>>(g->dg, R, y0, (const T *)r, scale, x, add);             \
+    else bp_slice_kernel<false, T><<<grid, 256, 0, st>>>(g->dg, R, y0, (const T *)r, scale, x, add);
+        if (rt == BSGD_F32) { SLICE_GO(float) }
+        else if (rt == BSGD_BF16) { SLICE_GO(__nv_bfloat16) }
+        else { SLICE_GO(__half) }
+#undef SLICE_GO
+        BSGD_CUDA(cudaGetLastError());
+    }
+    return BSGD_OK;
 }
 
 bsgd_status launch_column_change(const bsgd_geometry *g, const SolveDev &S, bsgd_dtype st_t,

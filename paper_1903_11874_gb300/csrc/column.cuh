@@ -55,17 +55,27 @@ __device__ __forceinline__ float column_weight(const DeviceGeom &G, float len2, 
 // Detector columns whose lines may cross the unit cell centred at (px, py)
 // (voxel units from the volume's low corner): the shadow of the centre, widened
 // by a bound on the shadow of the half diagonal. cell_interval decides.
+template <bool kParallel = false>
 __device__ __forceinline__ int2 cell_columns(const DeviceGeom &G, int a, float px, float py) {
     const float4 *p = reinterpret_cast<const float4 *>(G.rays + a);
     const float4 A = __ldg(p), B = __ldg(p + 1), C = __ldg(p + 2);   // p0 | pu c0 | cu
     const float rx = px - A.x, ry = py - A.y;
     const float ax = B.z - A.x, ay = B.w - A.y, cx = C.y, cy = C.z;
-    const float D = fmaf(rx, cy, -ry * cx);
-    const float hd = 0.5f * (fabsf(cx) + fabsf(cy)), hn = 0.5f * (fabsf(ax) + fabsf(ay));
-    const float room = fabsf(D) - hd;
-    if (!(room > 0.f)) return make_int2(0, G.nu - 1);
-    const float fu = __fdividef(-fmaf(rx, ay, -ry * ax), D);
-    const float w = __fdividef(fmaf(fabsf(fu), hd, hn), room) + 0.01f;
+    const float hn = 0.5f * (fabsf(ax) + fabsf(ay));
+    const float N = fmaf(rx, ay, -ry * ax);
+    float fu, w;
+    if (kParallel) {   // every line along (ax, ay), (cx, cy) apart
+        const float D = fmaf(cx, ay, -cy * ax);
+        fu = __fdividef(N, D);
+        w = __fdividef(hn, fabsf(D)) + 0.01f;
+    } else {
+        const float D = fmaf(rx, cy, -ry * cx);
+        const float hd = 0.5f * (fabsf(cx) + fabsf(cy));
+        const float room = fabsf(D) - hd;
+        if (!(room > 0.f)) return make_int2(0, G.nu - 1);
+        fu = __fdividef(-N, D);
+        w = __fdividef(fmaf(fabsf(fu), hd, hn), room) + 0.01f;
+    }
     const float uc = fu + 0.5f * (float)(G.nu - 1);
     const float lo = fminf(fmaxf(ceilf(uc - w), 0.f), (float)G.nu);
     const float hi = fmaxf(fminf(floorf(uc + w), (float)(G.nu - 1)), -1.f);

@@ -244,6 +244,7 @@ static void free_geometry(bsgd_geometry *g) {
     cudaFree(g->d_view_yfast);
     cudaFree(g->d_zoff);
     cudaFree(g->d_cray);
+    cudaFree(g->d_slice);
     for (int k = 0; k < 5; ++k) {
         cudaFree(g->d_counts[k]);
         cudaFree(g->d_cw[k]);

@@ -1170,6 +1170,8 @@ bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int 
         if (vT) BSGD_TRY(plain_transpose(g, v32, BSGD_F32, vT, j, j + 1, st));
         BSGD_TRY(launch_fp_plain(g, L, v32, BSGD_F32, y, BSGD_F32, 1, st, vT));
         if (cw) return launch_bp_column(g, L, y, BSGD_F32, w, 1.0f, 0, cw, st);
+        if (slice_bp_pays(g, g->plane_start[j + 1] - g->plane_start[j], views))
+            return launch_bp_slice(g, L, y, BSGD_F32, w, 1.0f, 0, st);
         if (wT) BSGD_CUDA(cudaMemsetAsync(wT + b0, 0, (b1 - b0) * 4, st));
         BSGD_TRY(launch_bp_plain(g, L, y, BSGD_F32, w, 1.0f, st, wT));
         if (wT) BSGD_TRY(plain_add_transposed(g, wT, w, j, j + 1, st));
@@ -1622,7 +1624,7 @@ size_t state_bytes(const bsgd_geometry_desc &d, int M, int N, const bsgd_solve_p
     b += 4 * (size_t)65536 * stride;                   // trace
     b += 8 * (size_t)N * d.n_views * cells * (p.cells == BSGD_CELLS_GEOMETRIC ? 2 : 1);
     // geometry tables
-    if (d.kind == BSGD_CONE3D && d.nz > 1 && d.nv > 1) b += sizeof(ColRay) * (size_t)d.n_views * d.nu;
+    if (d.kind != BSGD_CONE3D || (d.nz > 1 && d.nv > 1)) b += sizeof(ColRay) * (size_t)d.n_views * d.nu;
     b += 64 * (size_t)d.n_views + 16 * (size_t)d.n_views * (N + 1) + 4 * ((size_t)M * maxV + M + N + 1 + d.n_views);
     size_t t = 0;
     if (p.step_rule != BSGD_STEP_FIXED) t = std::max(t, C * 8 + R * 4 + C * 8 / N + 64);

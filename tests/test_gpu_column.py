@@ -66,6 +66,41 @@ def test_back_projection(name):
     assert torch.equal(x, again)
 
 
+SLICES = {
+    "par_odd": dict(kind="par2d", nx=67, ny=66, nz=1, dx=1.0, dy=1.0, dz=1.0, n_views=37, nu=101, nv=1,
+                    du=0.9, dv=1.0),
+    "par_bins_in_faces": dict(kind="par2d", nx=64, ny=64, nz=1, dx=1.0, dy=1.0, dz=1.0, n_views=4, nu=67,
+                              nv=1, du=1.0, dv=1.0),
+    "fan_coarse": dict(kind="fan2d", nx=96, ny=64, nz=1, dx=1.0, dy=1.5, dz=1.0, n_views=30, nu=40, nv=1,
+                       du=8.0, dv=1.0, dso=200.0, dsd=400.0),
+    "fan_fine": dict(kind="fan2d", nx=65, ny=70, nz=1, dx=1.2, dy=1.0, dz=1.0, n_views=9, nu=600, nv=1,
+                     du=0.5, dv=1.0, dso=150.0, dsd=300.0),
+}
+
+
+@pytest.mark.parametrize("name", list(SLICES))
+def test_slice_back_projection(name):
+    """2D images: the bounds of test_back_projection (ends of the rays up to 250
+    voxels from the corner; single rows of pixels scatter)."""
+    s = dict(SLICES[name], M=3, N=SLICES[name]["ny"])
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = torch.from_numpy(synth.normal_array(og.n_rows, 6)).to(DEV, torch.bfloat16)
+    x = torch.full((og.n_cols,), 3.0, device=DEV)
+    B.bsgd_back_project(gg, r, x)
+    got, r64 = x.cpu().double().numpy(), r.double().cpu().numpy()
+    assert rel_l2(got, P.bp(og, r64).reshape(-1)) <= 4e-5
+    thin = torch.zeros_like(x)
+    for j in range(gg.N):
+        B.bsgd_back_project(gg, r, thin, col_blocks=[j])
+    assert rel_l2(got, thin.cpu().double().numpy()) <= 2e-5
+    # two row blocks, scaled, added onto the image
+    y = x.clone()
+    B.bsgd_back_project(gg, r, y, row_blocks=[2, 0], scale=-2.0, accumulate=True)
+    rows = np.sort(np.concatenate([P.rows_of_views(og, P.row_block_views(og, 3, i)) for i in (0, 2)]))
+    ref = got - 2.0 * P.bp_rows(og, r64[rows], rows, None)
+    assert rel_l2(y.cpu().double().numpy(), ref) <= 4e-5
+
+
 def test_blocks_scale_accumulate_and_storage():
     """Two separate runs of slabs (the middle one on both sides of the source's
     height), some row blocks, added onto an image, from a BF16 residual."""
