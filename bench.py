@@ -44,19 +44,15 @@ UNIT = "GVox-ray/s"
 # the next crossing, the segment difference, the accumulate / weight product and
 # the recomputed crossing.
 ALU_OPS_PER_UPDATE = 5
-# DRAM bytes (read + write) per launch of the fused kernel, mean over the 64
-# launches of one epoch of this workload, from one ncu capture of the current
-# kernel (its DRAM-traffic capture is summarised under profiles/); null for the
-# split kernels, which were not captured.
-TRAFFIC_PER_LAUNCH = {"fpbp": 46_481_784}
-# What does bind the fused kernel, from the same kernel's ncu --set full capture
-# (the full capture summarised under profiles/, the heavier of two pairs):
-# L2 and L1/TEX throughput in % of their peaks, issue-active cycles in %, and
-# L1 -> L2 sector operations per voxel-ray update (FP + BP) and per BP update
-# (the reductions).
-ON_CHIP_NCU = {"fpbp": {"l2_pct": 64.6, "l1tex_pct": 68.3, "issue_active_pct": 46.8,
-                        "l2_sectors_per_update": 0.30, "red_sectors_per_bp_update": 0.51,
-                        "thread_instructions_per_update": 23.7}}
+# DRAM bytes (read + write) per pass, from an ncu capture of the current kernels;
+# null for passes that were not captured (the FP with the residual and the
+# gathering BP that now make up the fused pass).
+TRAFFIC_PER_LAUNCH = {}
+# What binds the passes on chip, from ncu captures of the current kernels
+# (summarised under profiles/): the gathering BP on one slab of this workload.
+ON_CHIP_NCU = {"fpbp": {"kernel": "bp_gather_kernel (the BP's half of the pass)", "l1tex_pct": 75.9,
+                        "issue_active_pct": 66.9, "warp_instructions_per_launch": 161_189_658,
+                        "updates_per_launch": 171_855_901}}
 
 
 # Serving workload: Poisson arrivals (20 / s), request sizes n^3 with (256 / n) mm
@@ -237,13 +233,14 @@ def algorithmic_bytes(gg, n_pairs_avg_rays, storage_bytes=4):
     z^j of the blocks whose band holds the ray (compact band storage; on
     average `nb` of them, from the geometry's band areas), and writes z^J and
     r; BP reads r and r~^J, writes r~^J and read-modify-writes g_J; the fused
-    kernel does both without re-reading r."""
+    pass does both without re-reading r and hands the BP its weights through
+    memory (written and read once)."""
     vox_j = gg.n_cols // N
     rays = n_pairs_avg_rays
     nb = max(1.0, gg.compact_rows / gg.n_rows)
     fp = vox_j * storage_bytes + rays * storage_bytes * (1 + nb + 1 + 2)
     bp = rays * storage_bytes * 3 + vox_j * 8
-    fpbp = vox_j * (storage_bytes + 8) + rays * storage_bytes * (nb + 6)
+    fpbp = vox_j * (storage_bytes + 8) + rays * (storage_bytes * (nb + 6) + 8)
     return {"fp": fp, "bp": bp, "fpbp": fpbp}
 
 
@@ -327,7 +324,7 @@ def run_cuda(args):
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     hbm_ach = dom_bytes / (launch_ms * 1e-3) / 1e9
     roofline = {
-        "bound": "alu", "kernel": "%s_solve_kernel" % dom,
+        "bound": "alu", "kernel": "fpbp_solve_kernel + solve_gather_kernel" if dom == "fpbp" else "%s_solve_kernel" % dom,
         "achieved": round(achieved, 3), "peak": round(alu_peak, 2),
         "unit": "T FP32-pipe instr/s (%d per update)" % ALU_OPS_PER_UPDATE,
         "frac": round(achieved / alu_peak, 4), "traffic": TRAFFIC_PER_LAUNCH.get(dom),
@@ -339,7 +336,8 @@ def run_cuda(args):
     }
     stages = {k: {"launches": v["launches"], "ms": round(v["ms"], 3)} for k, v in prof.items()
               if v["launches"]}
-    launches = sum(v["launches"] for v in prof.values())
+    # the fused pass of this workload, counted once, is two kernels
+    launches = sum(v["launches"] for v in prof.values()) + prof["fpbp"]["launches"]
 
     # ---- end to end through the public one-call API with host buffers
     e2e = None
@@ -405,7 +403,7 @@ def run_cuda(args):
                     "state_gb": round(B.bsgd_request_bytes(GEOM, M, N, prm) / 1e9, 3)},
             "gpu_launches": int(launches), "stages_ms": stages,
             "ms_per_step_profiled": round(ms_profiled / args.steps, 3),
-            "kernels": "split FP / BP" if args.split else "fused FP+residual+BP",
+            "kernels": "split FP / BP" if args.split else "FP with residual, gathering BP",
             "roofline": roofline, "clocks": clk, "e2e": e2e, "e2e_full_solve": full_solve,
             "cpu_baseline": cpu,
             "serving": serving, "paper_scale": paper, "rows": extra,
@@ -594,11 +592,11 @@ def update_leg(B, torch, dev, gg, y, mu, prof, hbm):
         st1.block_step(x1, 1)
     p1 = st1.read_profile()
     st1.close()
-    # a7: block update, 20 B per voxel of the slab (read x, g, gT; write x, xT)
+    # a7: block update, 16 B per voxel of the slab (read x, g; write x, xT)
     vox_j = gg.n_cols // N
     ms_u = p1["update"]["ms"] / max(p1["update"]["launches"], 1)
-    gbs = 20.0 * vox_j / (ms_u * 1e-3) / 1e9
-    out["a7_update"] = {"ms_per_launch": round(ms_u, 4), "bytes_per_launch": 20 * vox_j,
+    gbs = 16.0 * vox_j / (ms_u * 1e-3) / 1e9
+    out["a7_update"] = {"ms_per_launch": round(ms_u, 4), "bytes_per_launch": 16 * vox_j,
                         "achieved_gbs": round(gbs, 1), "peak_gbs": hbm, "frac": round(gbs / hbm, 4),
                         "bound": "hbm"}
     ms_s = p1["sample"]["ms"] / max(p1["sample"]["launches"], 1)
