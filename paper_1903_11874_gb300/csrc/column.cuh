@@ -55,8 +55,9 @@ __device__ __forceinline__ float column_weight(const DeviceGeom &G, float len2, 
 // Detector columns whose lines may cross the unit cell centred at (px, py)
 // (voxel units from the volume's low corner): the shadow of the centre, widened
 // by a bound on the shadow of the half diagonal. cell_interval decides.
+// t: ray parameter at the centre (divergent beams).
 template <bool kParallel = false>
-__device__ __forceinline__ int2 cell_columns(const DeviceGeom &G, int a, float px, float py) {
+__device__ __forceinline__ int2 cell_columns(const DeviceGeom &G, int a, float px, float py, float *t = nullptr) {
     const float4 *p = reinterpret_cast<const float4 *>(G.rays + a);
     const float4 A = __ldg(p), B = __ldg(p + 1), C = __ldg(p + 2);   // p0 | pu c0 | cu
     const float rx = px - A.x, ry = py - A.y;
@@ -70,6 +71,7 @@ __device__ __forceinline__ int2 cell_columns(const DeviceGeom &G, int a, float p
         w = __fdividef(hn, fabsf(D)) + 0.01f;
     } else {
         const float D = fmaf(rx, cy, -ry * cx);
+        if (t) *t = __fdividef(D, fmaf(ax, cy, -ay * cx));
         const float hd = 0.5f * (fabsf(cx) + fabsf(cy));
         const float room = fabsf(D) - hd;
         if (!(room > 0.f)) return make_int2(0, G.nu - 1);
@@ -223,6 +225,7 @@ __device__ __forceinline__ void gather_column(const DeviceGeom &G, int n_slots, 
     const int lane = threadIdx.x & 31, chunks = (z1 - z0 + 31) >> 5;
     const unsigned below = (1u << lane) - 1u;
     const float fx = (float)x - 0.5f * (float)G.nx, fy = (float)y - 0.5f * (float)G.ny;
+    const float ka = (float)z0 - G.zs, kb = (float)z1 - G.zs, vc = 0.5f * (float)(G.nv - 1);
     for (int q = 0; q < chunks; ++q) M.sums[q][lane] = 0.f;
 
     // the first m <= 32 candidates
@@ -271,7 +274,16 @@ __device__ __forceinline__ void gather_column(const DeviceGeom &G, int n_slots, 
     for (int b = 0; b < n_slots; b += 32) {
         int cell = -1, slot = b + lane, kd = 0;
         const int a = slot < n_slots ? view(slot, cell) : -1;
-        int2 ur = a >= 0 ? cell_columns(G, a, (float)x + 0.5f, (float)y + 0.5f) : make_int2(0, -1);
+        int2 ur = make_int2(0, -1);
+        if (a >= 0) {
+            float t;
+            ur = cell_columns(G, a, (float)x + 0.5f, (float)y + 0.5f, &t);
+            // nothing to do where all planes lie past the detector's rows (by the
+            // rows at the cell's centre and a bound on their change across it)
+            const float c = __fdividef(1.f, t * G.vstep), more = G.vslack * (1.f / 32.f);
+            const float top = fmaf(kb, c, fmaf(fabsf(kb), more, vc)), bottom = fmaf(ka, c, fmaf(-fabsf(ka), more, vc));
+            if (top < -0.5f || bottom > (float)G.nv - 0.5f) ur.y = -1;
+        }
         if (cell >= 0) {
             if (cell & 1) ur.x = max(ur.x, G.nu / 2);
             else ur.y = min(ur.y, G.nu / 2 - 1);
