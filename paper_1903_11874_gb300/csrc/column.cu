@@ -47,7 +47,7 @@ __global__ void column_tables_kernel(const DeviceGeom G, ColRay *__restrict__ cr
 // and the rise of its row j = v - (nv - 1) / 2 (the level row: j = 1), through a
 // 32 x 33 shared tile so that both sides are coalesced. Rows of nvp elements.
 template <typename T>
-__global__ void __launch_bounds__(256) column_weights_kernel(const DeviceGeom G, const RowSel R,
+__global__ void __launch_bounds__(256) column_weights_kernel(const DeviceGeom G, const RowSel R, int j0, int j1,
                                                              const T *__restrict__ r, float scale,
                                                              float *__restrict__ w) {
     __shared__ float s[32][33];
@@ -56,6 +56,10 @@ __global__ void __launch_bounds__(256) column_weights_kernel(const DeviceGeom G,
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int tu = (G.nu + 31) / 32;
     const int u0 = (blockIdx.x % tu) * 32, v0 = (int)(blockIdx.x / tu) * 32 - G.vpad;
+    // rays outside the slab's band meet none of its voxels: their weights are not
+    // read as data; the padding, whose rows could, is always written
+    const Band b = band_of(G, a, j0, j1);
+    if (v0 >= 0 && v0 + 32 <= G.nv && (u0 > b.u1 || u0 + 31 < b.u0 || v0 > b.v1 || v0 + 31 < b.v0)) return;
     const ColRay C = load_ray(G.cray + (size_t)a * G.nu + min(u0 + lane, G.nu - 1));
     const float len = column_length2(G, C);
 #pragma unroll
@@ -310,9 +314,9 @@ bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const
         R.n = std::min(64, L.n_rb - k);
         for (int t = 0; t < R.n; ++t) R.ids[t] = L.row_ids[k + t];
         const dim3 wg((unsigned)((g->desc.nu + 31) / 32 * ((g->dg.nvp + 31) / 32)), R.n * g->max_views);
-        if (rt == BSGD_F32) column_weights_kernel<float><<<wg, 256, 0, st>>>(g->dg, R, (const float *)r, scale, w);
-        else if (rt == BSGD_BF16) column_weights_kernel<__nv_bfloat16><<<wg, 256, 0, st>>>(g->dg, R, (const __nv_bfloat16 *)r, scale, w);
-        else column_weights_kernel<__half><<<wg, 256, 0, st>>>(g->dg, R, (const __half *)r, scale, w);
+        if (rt == BSGD_F32) column_weights_kernel<float><<<wg, 256, 0, st>>>(g->dg, R, L.j0, L.j1, (const float *)r, scale, w);
+        else if (rt == BSGD_BF16) column_weights_kernel<__nv_bfloat16><<<wg, 256, 0, st>>>(g->dg, R, L.j0, L.j1, (const __nv_bfloat16 *)r, scale, w);
+        else column_weights_kernel<__half><<<wg, 256, 0, st>>>(g->dg, R, L.j0, L.j1, (const __half *)r, scale, w);
         bp_gather_kernel<<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, R, z0, z1, w, x, accumulate || k > 0);
         BSGD_CUDA(cudaGetLastError());
     }
