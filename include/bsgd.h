@@ -487,9 +487,9 @@ bsgd_status bsgd_state_read_profile(bsgd_state *s, bsgd_profile *out, void *stre
  * bsgd_state_restore: loads a checkpoint into s, a state created from the same
  *   geometry, parameters and y (a fresh one, or the same one to roll back);
  *   continue with bsgd_block_step and the x of the save. Restores the
- *   sampling mode the saved state ran with (bsgd_state_set_sampling). A blob of
- *   a state that scattered (with a y-fastest part of g) restores into one that
- *   gathers. Synchronises `stream`. Errors: INVALID_ARG when the blob is not a
+ *   sampling mode the saved state ran with (bsgd_state_set_sampling). States that
+ *   scatter (their g has a y-fastest part) and states that gather take each
+ *   other's blobs. Synchronises `stream`. Errors: INVALID_ARG when the blob is not a
  *   checkpoint of a state of this geometry, block counts, pair counts and
  *   storage type, or is truncated.
  */

@@ -1999,11 +1999,9 @@ struct CkptPart {
     size_t bytes;
 };
 
-constexpr size_t kCkptTracePart = 9;   // the trace is the ninth part
-
 // The device arrays of a checkpoint, in blob order; trace rows = iterations
-// recorded so far.
-std::vector<CkptPart> ckpt_parts(const bsgd_state *s, int64_t trace_rows) {
+// recorded so far. gT: the y-fastest part of g, null in a blob whose g is whole.
+std::vector<CkptPart> ckpt_parts(const bsgd_state *s, int64_t trace_rows, float *gT) {
     const bsgd_geometry *g = s->g;
     const size_t es = dtype_size(s->st), R = (size_t)g->n_rows(), C = (size_t)g->n_cols();
     const size_t Z = (size_t)g->zlen;
@@ -2011,7 +2009,7 @@ std::vector<CkptPart> ckpt_parts(const bsgd_state *s, int64_t trace_rows) {
         {s->z, Z * es}, {s->rt, Z * es}, {s->r, R * es}, {s->grad, C * 4},
         {s->S, 8 * (size_t)g->M * g->desc.nv}, {s->d_mu, 8}, {s->d_iter, 8}, {s->updates, 8},
         {s->trace, 4 * (size_t)trace_rows * s->stride}};
-    if (s->gT) v.push_back({s->gT, C * 4});
+    if (gT) v.push_back({gT, C * 4});
     if (s->xlo) v.push_back({s->xlo, C * es});
     if (s->eud) {
         v.push_back({s->eud, 8 * C});
@@ -2019,6 +2017,12 @@ std::vector<CkptPart> ckpt_parts(const bsgd_state *s, int64_t trace_rows) {
         v.push_back({s->am, sizeof(AutoMuHist)});
     }
     return v;
+}
+
+size_t ckpt_bytes(const std::vector<CkptPart> &parts) {
+    size_t n = 0;
+    for (const CkptPart &q : parts) n += q.bytes;
+    return n;
 }
 
 CkptHeader ckpt_header(const bsgd_state *s) {
@@ -2043,9 +2047,7 @@ CkptHeader ckpt_header(const bsgd_state *s) {
     h.iters = s->iters;
     h.trace_rows = std::min(s->iters, s->trace_cap);
     h.seed = s->p.seed;
-    size_t tot = 0;
-    for (const CkptPart &q : ckpt_parts(s, h.trace_rows)) tot += q.bytes;
-    h.payload = (int64_t)tot;
+    h.payload = (int64_t)ckpt_bytes(ckpt_parts(s, h.trace_rows, s->gT));
     return h;
 }
 
@@ -2066,7 +2068,7 @@ extern "C" bsgd_status bsgd_state_save(bsgd_state *s, void *host, int64_t cap, v
     char *out = static_cast<char *>(host);
     std::memcpy(out, &h, sizeof h);
     size_t off = sizeof h;
-    for (const CkptPart &q : ckpt_parts(s, h.trace_rows)) {
+    for (const CkptPart &q : ckpt_parts(s, h.trace_rows, s->gT)) {
         if (q.bytes) BSGD_CUDA(cudaMemcpyAsync(out + off, q.dev, q.bytes, cudaMemcpyDeviceToHost, st));
         off += q.bytes;
     }
@@ -2090,37 +2092,31 @@ extern "C" bsgd_status bsgd_state_restore(bsgd_state *s, const void *host, int64
         return fail(BSGD_ERR_INVALID_ARG, "checkpoint of a different geometry or solver set-up");
     if (h.iters < 0 || h.trace_rows != std::min(h.iters, s->trace_cap))
         return fail(BSGD_ERR_INVALID_ARG, "corrupt checkpoint header");
-    const std::vector<CkptPart> parts = ckpt_parts(s, h.trace_rows);
-    size_t need = 0;
-    for (const CkptPart &q : parts) need += q.bytes;
-    // a state that scattered kept part of g y-fastest, after the trace
-    const size_t C = (size_t)s->g->n_cols();
-    const bool old_gT = s->w && (int64_t)(need + C * 4) == h.payload;
-    if (old_gT) need += C * 4;
-    if ((int64_t)need != h.payload || bytes < (int64_t)sizeof(CkptHeader) + h.payload)
+    // a state that scatters keeps part of g y-fastest and one that gathers does
+    // not; either takes the other's blob
+    const int64_t whole = (int64_t)ckpt_bytes(ckpt_parts(s, h.trace_rows, nullptr));
+    const int64_t split = whole + s->g->n_cols() * 4;
+    if (!(h.payload == whole || h.payload == split) || (!s->gT && !s->w && h.payload != whole) ||
+        bytes < (int64_t)sizeof(CkptHeader) + h.payload)
         return fail(BSGD_ERR_INVALID_ARG, "checkpoint truncated");
     cudaStream_t st = (cudaStream_t)stream;
     if (h.pair_sampling != s->p.pair_sampling || h.cells != s->p.cells || h.n_cells != s->n_cells)
         BSGD_TRY(bsgd_state_set_sampling(s, h.pair_sampling, h.cells, h.n_cells, stream));
-    float *gT = nullptr;
-    if (old_gT) BSGD_TRY(palloc((void **)&gT, C * 4, st));
+    float *own = nullptr;   // the blob's gT for a state without one
+    if (h.payload == split && !s->gT) BSGD_TRY(palloc((void **)&own, s->g->n_cols() * 4, st));
     auto load = [&]() -> bsgd_status {
         const char *in = static_cast<const char *>(host) + sizeof h;
-        for (size_t k = 0; k < parts.size(); ++k) {
-            const CkptPart &q = parts[k];
+        for (const CkptPart &q : ckpt_parts(s, h.trace_rows, h.payload == whole ? nullptr : own ? own : s->gT)) {
             if (q.bytes) BSGD_CUDA(cudaMemcpyAsync(q.dev, in, q.bytes, cudaMemcpyHostToDevice, st));
             in += q.bytes;
-            if (gT && k + 1 == kCkptTracePart) {
-                BSGD_CUDA(cudaMemcpyAsync(gT, in, C * 4, cudaMemcpyHostToDevice, st));
-                BSGD_TRY(plain_add_transposed(s->g, gT, s->grad, 0, s->g->N, st));
-                in += C * 4;
-            }
         }
+        if (own) BSGD_TRY(plain_add_transposed(s->g, own, s->grad, 0, s->g->N, st));
+        if (s->gT && h.payload == whole) BSGD_CUDA(cudaMemsetAsync(s->gT, 0, s->g->n_cols() * 4, st));
         BSGD_CUDA(cudaStreamSynchronize(st));
         return BSGD_OK;
     };
     const bsgd_status le = load();
-    pool_free(gT, st);
+    pool_free(own, st);
     BSGD_TRY(le);
     s->iters = h.iters;
     cudaFree(s->replay);   // a replay in progress belongs to the state that was replaced

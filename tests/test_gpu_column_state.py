@@ -1,0 +1,107 @@
+"""Solver states around the gathering back projection: checkpoints between a
+state that gathers and one that scatters."""
+import struct
+
+import numpy as np
+import pytest
+
+from helpers import gpu_geom, oracle_geom, rel_l2
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import projector as P  # noqa: E402
+from paper_1903_11874_gb300 import binding as B  # noqa: E402
+from paper_1903_11874_gb300 import synth  # noqa: E402
+
+DEV = "cuda:0"
+
+
+def solve_geometry(kN, **over):
+    """The smallest size whose solver gathers; odd nv, uneven slabs (one block)."""
+    M = 1 if kN == 1 else 2
+    s = dict(kind="cone3d", nx=128, ny=126, nz=63 if kN == 1 else 64, dx=1.0, dy=1.0, dz=1.0, n_views=52,
+             nu=110, nv=71, du=2.2, dv=2.2, dso=300.0, dsd=600.0, M=M, N=2)
+    s.update(over)
+    return s
+
+
+def scan(og, s):
+    xt = synth.ellipsoid_phantom(s["nx"], s["ny"], s["nz"], 4, seed=1).reshape(-1).astype(np.float64) * 0.01
+    return P.fp(og, xt).reshape(-1).astype(np.float32)
+
+
+@pytest.fixture(scope="module")
+def one_block():
+    s = solve_geometry(1)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    return gg, torch.from_numpy(scan(og, s)).to(DEV)
+
+
+def one_block_state(one_block, cells):
+    gg, y = one_block
+    prm = B.SolveParams(alpha=1.0, gamma=0.5, step_rule=B.STEP_FIXED, mu=2e-5, seed=5, cells=cells,
+                        n_cells=1 if cells == B.CELLS_NONE else 4)
+    return B.State(gg, prm, y)
+
+
+def run_on(st, x, n):
+    st.block_step(x, n)
+    return x.cpu().double().numpy()
+
+
+@pytest.mark.parametrize("first,second", [(B.CELLS_NONE, B.CELLS_GEOMETRIC), (B.CELLS_GEOMETRIC, B.CELLS_NONE)])
+def test_checkpoint_between_sampling_modes(one_block, first, second):
+    """A state created with whole views gathers, one created with detector cells
+    scatters; a blob of either continues in the other.
+
+    Bound: both runs are the same iterations in FP32, each within 1e-5 of the
+    exact image (the parity bound of the solver tests): 2e-5 between them."""
+    a, b = one_block_state(one_block, first), one_block_state(one_block, second)
+    x = torch.zeros(one_block[0].n_cols, device=DEV)
+    a.block_step(x, 4)
+    blob, xb = a.save(), x.clone()
+    b.restore(blob)
+    assert b.query()["residual_norm"] == a.query()["residual_norm"]
+    assert rel_l2(run_on(b, xb, 3), run_on(a, x, 3)) <= 2e-5
+
+
+def split_blob(blob, gg, whole):
+    """The blob with g moved wholly into its y-fastest part (whole = False), or
+    such a blob with that part added back."""
+    payload = struct.unpack_from("<q", blob, 128)[0]
+    at, C = 144 + 4 * (2 * gg.compact_rows + gg.n_rows), gg.n_cols
+    shape = (gg.nz, gg.ny, gg.nx)
+    head, g, rest = bytearray(blob[:at]), np.frombuffer(blob, np.float32, C, at).reshape(shape), blob[at + 4 * C:]
+    if whole:
+        gT = np.frombuffer(rest[-4 * C:], np.float32).reshape(gg.nz, gg.nx, gg.ny)
+        struct.pack_into("<q", head, 128, payload - 4 * C)
+        return bytes(head) + (g + gT.transpose(0, 2, 1)).astype(np.float32).tobytes() + rest[:-4 * C]
+    struct.pack_into("<q", head, 128, payload + 4 * C)
+    return bytes(head) + bytes(4 * C) + rest + np.ascontiguousarray(g.transpose(0, 2, 1)).tobytes()
+
+
+def test_checkpoint_with_and_without_the_y_fastest_gradient(one_block):
+    """A state that gathers takes the blob of one that scatters with the same
+    parameters (part of g stored y-fastest, after the trace), and the other way
+    round; a blob cut short stays refused."""
+    gg, _ = one_block
+    a = one_block_state(one_block, B.CELLS_NONE)
+    x = torch.zeros(gg.n_cols, device=DEV)
+    a.block_step(x, 4)
+    blob, xb = a.save(), x.clone()
+    ref = run_on(a, x, 3)
+    b = one_block_state(one_block, B.CELLS_NONE)
+    b.restore(split_blob(blob, gg, False))
+    assert np.array_equal(run_on(b, xb.clone(), 3), ref)   # the same g, and the gather is reproducible
+    c = one_block_state(one_block, B.CELLS_GEOMETRIC)
+    xc = torch.zeros(gg.n_cols, device=DEV)
+    c.block_step(xc, 4)
+    cblob, xd = c.save(), xc.clone()
+    ref = run_on(c, xc, 3)
+    d = one_block_state(one_block, B.CELLS_GEOMETRIC)
+    d.restore(split_blob(cblob, gg, True))
+    assert rel_l2(run_on(d, xd, 3), ref) <= 2e-5
+    for bad in (blob[:-4], split_blob(blob, gg, False)[:-4]):
+        with pytest.raises(B.BSGDError):
+            b.restore(bad)
