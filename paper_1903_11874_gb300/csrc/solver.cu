@@ -1320,14 +1320,34 @@ static bsgd_status geometry_tables(const bsgd_geometry *g, int n_cells, bool wei
     return BSGD_OK;
 }
 
+static bsgd_status create_form(const bsgd_geometry *g, const bsgd_solve_params *p, const void *y,
+                               bsgd_dtype yt, bool column, cudaStream_t st, bsgd_state **out,
+                               bool *gathers);
+
 extern "C" bsgd_status bsgd_state_create(const bsgd_geometry *g, const bsgd_solve_params *p,
                                          const void *y, bsgd_dtype yt, void *stream,
                                          bsgd_state **out) {
     return state_create(g, p, y, yt, true, (cudaStream_t)stream, out);
 }
 
+// The weights of the gathering BP may be larger than the y-fastest gradient that
+// they replace: a set-up that runs out of memory with them is made without.
 bsgd_status bsgd::state_create(const bsgd_geometry *g, const bsgd_solve_params *p, const void *y,
                                bsgd_dtype yt, bool column, cudaStream_t st, bsgd_state **out) {
+    bool gathers = false;
+    bsgd_status e = create_form(g, p, y, yt, column, st, out, &gathers);
+    if (e == BSGD_ERR_OOM && gathers) {
+        cudaMemPool_t pool = nullptr;   // the first try's memory goes back first
+        cudaStreamSynchronize(0);
+        if (state_pool(&pool) == BSGD_OK) cudaMemPoolTrimTo(pool, 0);
+        e = create_form(g, p, y, yt, false, st, out, &gathers);
+    }
+    return e;
+}
+
+static bsgd_status create_form(const bsgd_geometry *g, const bsgd_solve_params *p, const void *y,
+                               bsgd_dtype yt, bool column, cudaStream_t st, bsgd_state **out,
+                               bool *gathers) {
     if (!g || !p || !y || !out) return fail(BSGD_ERR_INVALID_ARG, "NULL argument");
     *out = nullptr;
     if (!dtype_ok(yt)) return fail(BSGD_ERR_INVALID_ARG, "bad y dtype");
@@ -1359,10 +1379,7 @@ bsgd_status bsgd::state_create(const bsgd_geometry *g, const bsgd_solve_params *
     const int N = g->N, M = g->M, V = g->desc.n_views;
     bsgd_status e = BSGD_OK;
     const int64_t Z = g->zlen;   // compact band storage of z^j and r~^j
-    // column form: the BP gathers from weights that the FP leaves; without room
-    // for them the state scatters
     const size_t W = column ? column_solve_len(g, s->kM, s->kN, p->cells != BSGD_CELLS_NONE) : 0;
-    if (W) pool_try_alloc((void **)&s->w, W * 4, st);
     if ((e = palloc(&s->y, R * es, st)) || (e = palloc(&s->z, (size_t)Z * es, st)) ||
         (e = palloc(&s->rt, (size_t)Z * es, st)) || (e = palloc(&s->r, R * es, st)) ||
         (e = palloc((void **)&s->grad, C * 4, st)) || (e = palloc((void **)&s->S, 8 * (size_t)M * g->desc.nv, st)) ||
@@ -1377,16 +1394,20 @@ bsgd_status bsgd::state_create(const bsgd_geometry *g, const bsgd_solve_params *
         (e = palloc((void **)&s->pair_upd, 8 * (size_t)M * N, st)) ||
         (s->st != BSGD_F32 && !p->image_plain && (e = palloc(&s->xlo, C * es, st))) ||
         (g->desc.nz > 1 && (e = palloc(&s->xT, C * es, st))) ||
-        (g->desc.nz > 1 && !s->w && (e = palloc((void **)&s->gT, C * 4, st))) ||
         (p->tv_lambda > 0 && (e = tv_work_alloc(g, s->tv))) ||
         (p->auto_mu && ((e = palloc((void **)&s->eud, 8 * (size_t)C, st)) ||
                         (e = palloc((void **)&s->eud_prev, 8 * (size_t)C, st)) ||
                         (e = palloc((void **)&s->am_part, 8 * 3 * (size_t)kAutoParts, st)) ||
-                        (e = palloc((void **)&s->am, sizeof(AutoMuHist), st))))) {
+                        (e = palloc((void **)&s->am, sizeof(AutoMuHist), st)))) ||
+        // column form: the BP gathers from weights that the FP leaves, taken after
+        // all that the state cannot do without; without room for them it scatters
+        (!(W && pool_try_alloc((void **)&s->w, W * 4, st)) && g->desc.nz > 1 &&
+         (e = palloc((void **)&s->gT, C * 4, st)))) {
         cudaStreamSynchronize(st);
         free_state(s);
         return e;
     }
+    *gathers = s->w != nullptr;
     auto init = [&]() -> bsgd_status {
         BSGD_TRY(convert(y, yt, s->y, s->st, R, st));
         BSGD_CUDA(cudaMemcpyAsync(s->r, s->y, R * es, cudaMemcpyDeviceToDevice, st));
@@ -2212,12 +2233,13 @@ extern "C" bsgd_status bsgd_solve(const bsgd_geometry *g, const bsgd_solve_param
             BSGD_CUDA(cudaMemcpyAsync(dy, y, R * dtype_size(yt), cudaMemcpyHostToDevice, st));
             yy = dy;
         }
-        BSGD_TRY(bsgd_state_create(g, p, yy, yt, stream, &s));
+        // the images before the state, whose optional memory takes what is left
         const bsgd_dtype sd = (bsgd_dtype)p->storage;
         BSGD_TRY(palloc(&xs, C * dtype_size(sd), st));
+        if (xh) BSGD_TRY(palloc(&dx, C * dtype_size(xt), st));
+        BSGD_TRY(bsgd_state_create(g, p, yy, yt, stream, &s));
         // x holds the starting image x0 (the first block step warm-starts from
         // it) unless the caller asks for Algorithm 1's zero start
-        if (xh) BSGD_TRY(palloc(&dx, C * dtype_size(xt), st));
         if (p->zero_start) {
             BSGD_CUDA(cudaMemsetAsync(xs, 0, C * dtype_size(sd), st));
             s->zero_start = true;   // the state already describes x0 = 0

@@ -1,6 +1,9 @@
 """Solver states around the gathering back projection: checkpoints between a
-state that gathers and one that scatters."""
+state that gathers and one that scatters, and the memory that a state needs."""
+import os
 import struct
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -105,3 +108,37 @@ def test_checkpoint_with_and_without_the_y_fastest_gradient(one_block):
     for bad in (blob[:-4], split_blob(blob, gg, False)[:-4]):
         with pytest.raises(B.BSGDError):
             b.restore(bad)
+
+
+LITTLE_MEMORY = """
+import torch
+from helpers import gpu_geom
+from paper_1903_11874_gb300 import binding as B
+geo = dict(kind="cone3d", nx=128, ny=128, nz=64, dx=1.0, dy=1.0, dz=1.0, n_views=720, nu=512, nv=448,
+           du=1.6, dv=1.6, dso=300.0, dsd=600.0)
+gg = B.Geometry(M=1, N=2, **geo)
+y = torch.ones(gg.n_rows, device="cuda:0")
+prm = B.SolveParams(alpha=1.0, gamma=1.0, step_rule=B.STEP_FIXED, mu=1e-6, seed=5)
+x = torch.zeros(gg.n_cols, device="cuda:0")
+need = B.bsgd_request_bytes(geo, 1, 2, prm)
+torch.cuda.empty_cache()
+free = torch.cuda.mem_get_info()[0]
+hold = torch.empty(free - need - (1 << 28), dtype=torch.uint8, device="cuda:0")
+st = B.State(gg, prm, y)
+st.block_step(x, 1)
+torch.cuda.synchronize()
+assert bool(torch.isfinite(x).all()) and float(x.abs().max()) > 0
+st.close()
+B.bsgd_solve(gg, B.SolveParams(alpha=1.0, gamma=1.0, step_rule=B.STEP_FIXED, mu=1e-6, seed=5, epochs=1), y, x)
+print("MADE")
+"""
+
+
+def test_little_memory_scatters():
+    """With a gigabyte more than a scattering state holds, less than the 1.7 GB of
+    weights that the gather would take, the state is made and steps."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([here, os.path.dirname(here)]))
+    res = subprocess.run([sys.executable, "-c", LITTLE_MEMORY], cwd=os.path.dirname(here), env=env,
+                         capture_output=True, text=True, timeout=300)
+    assert "MADE" in res.stdout, res.stderr[-2000:]
