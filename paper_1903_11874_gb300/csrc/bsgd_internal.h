@@ -95,6 +95,7 @@ struct DeviceGeom {
     const float2 *sx, *sy;     // {xh, xl}, {yh, yl}
     const float2 *si;          // {ix, iy}
     const float *slen;         // length of the ray (mm)
+    float umargin;             // columns (column.cuh, cell_columns)
     float tc;                  // ray parameter of the rotation axis
     float zs;                  // source height (voxels from the volume's low face)
     float vstep;               // z slope per detector row

@@ -54,7 +54,8 @@ __device__ __forceinline__ float column_weight(const DeviceGeom &G, float len2, 
 
 // Detector columns whose lines may cross the unit cell centred at (px, py)
 // (voxel units from the volume's low corner): the shadow of the centre, widened
-// by a bound on the shadow of the half diagonal. cell_interval decides.
+// by a bound on the shadow of the half diagonal and by G.umargin, which holds the
+// rounding of the lines and of the shadow. cell_interval decides.
 // t: ray parameter at the centre (divergent beams).
 template <bool kParallel = false>
 __device__ __forceinline__ int2 cell_columns(const DeviceGeom &G, int a, float px, float py, float *t = nullptr) {
@@ -68,7 +69,7 @@ __device__ __forceinline__ int2 cell_columns(const DeviceGeom &G, int a, float p
     if (kParallel) {   // every line along (ax, ay), (cx, cy) apart
         const float D = fmaf(cx, ay, -cy * ax);
         fu = __fdividef(N, D);
-        w = __fdividef(hn, fabsf(D)) + 0.01f;
+        w = __fdividef(hn, fabsf(D)) + G.umargin;
     } else {
         const float D = fmaf(rx, cy, -ry * cx);
         if (t) *t = __fdividef(D, fmaf(ax, cy, -ay * cx));
@@ -76,7 +77,7 @@ __device__ __forceinline__ int2 cell_columns(const DeviceGeom &G, int a, float p
         const float room = fabsf(D) - hd;
         if (!(room > 0.f)) return make_int2(0, G.nu - 1);
         fu = __fdividef(-N, D);
-        w = __fdividef(fmaf(fabsf(fu), hd, hn), room) + 0.01f;
+        w = __fdividef(fmaf(fabsf(fu), hd, hn), room) + G.umargin;
     }
     const float uc = fu + 0.5f * (float)(G.nu - 1);
     const float lo = fminf(fmaxf(ceilf(uc - w), 0.f), (float)G.nu);

@@ -1,5 +1,5 @@
 """The gathering back projections where their work is dealt or declined: views of
-many small row blocks."""
+many small row blocks, and sources far away."""
 import numpy as np
 import pytest
 
@@ -41,3 +41,36 @@ def test_slice_views_dealt_over_all_blocks(views, M, block):
     again = torch.zeros_like(got)
     B.bsgd_back_project(gpu_geom(s), r, again)
     assert torch.equal(again, got)
+
+
+FAR = {
+    "cone_3e5": dict(kind="cone3d", nx=64, ny=64, nz=40, dx=1.0, dy=1.0, dz=1.0, n_views=6, nu=70, nv=45, du=2.0,
+                     dv=2.0, dso=3e5, dsd=6e5),
+    "cone_1e6": dict(kind="cone3d", nx=64, ny=64, nz=40, dx=1.0, dy=1.0, dz=1.0, n_views=6, nu=70, nv=45, du=2.0,
+                     dv=2.0, dso=1e6, dsd=2e6),
+    "cone_1e7": dict(kind="cone3d", nx=64, ny=64, nz=40, dx=1.0, dy=1.0, dz=1.0, n_views=6, nu=70, nv=45, du=2.0,
+                     dv=2.0, dso=1e7, dsd=2e7),
+    "fan_1e6": dict(kind="fan2d", nx=70, ny=70, nz=1, dx=1.0, dy=1.0, dz=1.0, n_views=30, nu=300, nv=1, du=0.5,
+                    dv=1.0, dso=1e6, dsd=2e6),
+}
+
+
+@pytest.mark.parametrize("name", list(FAR))
+def test_far_sources_lose_no_ray(name):
+    """The sum over the volume is that of the oracle: no voxel misses a ray.
+
+    Bound: a ray's ends round to half an ulp of the source's distance, which moves
+    its length in the volume by up to four times that, either way: five standard
+    deviations of the mean over the rays, against their mean length. Rays past FP32
+    (1e7) are held to a tenth. The cones here lie beyond the gather's rule."""
+    s = dict(FAR[name], M=1, N=1)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = synth.uniform_array(og.n_rows, 3).astype(np.float32)
+    x = torch.zeros(og.n_cols, device=DEV)
+    B.bsgd_back_project(gg, torch.from_numpy(r).to(DEV), x)
+    chords = P.fp(og, np.ones(og.n_cols)).reshape(-1)
+    n, mean = int((chords > 0).sum()), chords.sum() / (chords > 0).sum()
+    ulp = float(np.spacing(np.float32(s["dso"])))
+    bound = 0.1 if s["dso"] > 5e6 else 5 * 4 * 0.5 * ulp / mean / np.sqrt(n)
+    ref = P.bp(og, r.astype(np.float64)).sum()
+    assert abs(x.double().sum().item() / ref - 1) <= bound
