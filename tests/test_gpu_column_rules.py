@@ -74,3 +74,53 @@ def test_far_sources_lose_no_ray(name):
     bound = 0.1 if s["dso"] > 5e6 else 5 * 4 * 0.5 * ulp / mean / np.sqrt(n)
     ref = P.bp(og, r.astype(np.float64)).sum()
     assert abs(x.double().sum().item() / ref - 1) <= bound
+
+
+def cone(n, nz, views, nu, nv, pitch, dso, mag, N):
+    return dict(kind="cone3d", nx=n, ny=n, nz=nz, dx=1.0, dy=1.0, dz=1.0, n_views=views, nu=nu, nv=nv, du=pitch,
+                dv=pitch, dso=dso, dsd=mag * dso, M=1, N=N)
+
+
+@pytest.mark.parametrize("nz,nv", [(48, 76), (48, 77), (49, 76), (32, 61), (20, 40)])
+def test_chunks_on_both_sides_of_a_near_source(nz, nv):
+    """Planes below and above the source's height in one chunk of 32, with the
+    source 11 voxels from the volume (rows per voxel change by up to 0.6 across a cell
+    there): level rows in a face, inside a voxel, and none. The bounds are those
+    of the plain gather's tests, against the oracle and the walk (thin blocks)."""
+    s = cone(60, nz, 9, 70, nv, 1.8, 54.0, 2.0, nz)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = synth.normal_array(og.n_rows, 3).astype(np.float32)
+    rd = torch.from_numpy(r).to(DEV)
+    x, thin = torch.zeros(og.n_cols, device=DEV), torch.zeros(og.n_cols, device=DEV)
+    B.bsgd_back_project(gg, rd, x)
+    for j in range(nz):
+        B.bsgd_back_project(gg, rd, thin, col_blocks=[j])
+    got = x.cpu().double().numpy()
+    assert rel_l2(got, P.bp(og, r.astype(np.float64)).reshape(-1)) <= 4e-5
+    assert rel_l2(got, thin.cpu().double().numpy()) <= 2e-5
+
+
+def time_of(f):
+    times = []
+    f()
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(4):
+            f()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    return sorted(times)[3]
+
+
+def test_near_source_chunk_costs_its_rows():
+    """One chunk on both sides of the source's height takes no more than twice its
+    two halves by themselves (seven times where every crossing took the rows that
+    the cell nearest to the source needs)."""
+    s = cone(128, 32, 60, 128, 128, 1.6, 100.0, 2.0, 2)
+    gg = gpu_geom(s)
+    r, x = torch.ones(gg.n_rows, device=DEV), torch.zeros(gg.n_cols, device=DEV)
+    whole = time_of(lambda: B.bsgd_back_project(gg, r, x))
+    halves = sum(time_of(lambda: B.bsgd_back_project(gg, r, x, col_blocks=[j])) for j in (0, 1))
+    assert whole <= 2.0 * halves
