@@ -265,9 +265,18 @@ static double gather_waste(const bsgd_geometry *g, int planes) {
 // us; 48 x 48 x 32 from 24 views 35 and 23 us; 32^3 from 90 views 35 and 39 us.
 // Full chunks gather 2.1 times as fast as they scatter at a waste of 0.8, 1.2
 // times at 1.4.
+// The padding of the weights measures a source that all but touches the volume
+// (rows per voxel that change across a cell by many rows, times the planes), where
+// a lane runs through the rows of the chunk's outermost plane; us scattered /
+// gathered with the padding per voxel of a view's weights in brackets: 128^3 from
+// 60 views, source 5.5 voxels away [0.29] 731 / 462, 3.5 [0.62] 726 / 630, 2.5 [1.1]
+// 756 / 818; 256^3 from 45, 4 voxels [0.40] 3771 / 3285, 3 [0.69] 3799 / 4298; a
+// 32-plane slab of it, 9 voxels [0.77] 769 / 585, 5 [2.1] 804 / 1243.
 bool column_bp_pays(const bsgd_geometry *g, int planes, int views) {
-    const int64_t voxels = (int64_t)g->desc.nx * g->desc.ny * planes;
-    return g->dg.nvp > 0 && planes > 0 && voxels >= (views <= 32 ? 64000 : 160000) && gather_waste(g, planes) <= 1.7;
+    const int64_t plane = (int64_t)g->desc.nx * g->desc.ny, voxels = plane * planes;
+    if (g->dg.nvp == 0 || planes <= 0 || voxels < (views <= 32 ? 64000 : 160000)) return false;
+    const double pad = (double)g->desc.nu * 2.0 * g->dg.vpad;
+    return pad <= 0.64 * (double)(plane * g->desc.nz) && pad <= 1.2 * (double)voxels && gather_waste(g, planes) <= 1.7;
 }
 
 static bsgd_status fill_tables(bsgd_geometry *g, bool slice) {

@@ -124,3 +124,36 @@ def test_near_source_chunk_costs_its_rows():
     whole = time_of(lambda: B.bsgd_back_project(gg, r, x))
     halves = sum(time_of(lambda: B.bsgd_back_project(gg, r, x, col_blocks=[j])) for j in (0, 1))
     assert whole <= 2.0 * halves
+
+
+def kernels_of(f):
+    """Names of the kernels that a call launches."""
+    f()
+    torch.cuda.synchronize()
+    for _ in range(3):   # (a process's first profile comes back empty)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            f()
+            torch.cuda.synchronize()
+        names = " ".join(e.key for e in prof.key_averages())
+        if "kernel" in names:
+            break
+    return names
+
+
+@pytest.mark.parametrize("dso,block,gathers", [(93.0, None, False), (96.0, None, True), (250.0, None, True),
+                                               (92.0, 1, False), (100.0, 1, True)])
+def test_sources_that_touch_the_volume_scatter(dso, block, gathers):
+    """The rule on the padding of the weights: the back projection from a source 2.5
+    voxels from the volume takes the walk, from 5.5 voxels the gather; either agrees
+    with the oracle (one view: the bound of the plain gather's tests)."""
+    s = cone(128, 128, 40, 128, 128, 1.6, dso, 2.0, 4)
+    og, gg = oracle_geom(dict(s, n_views=1)), gpu_geom(s)
+    r = np.zeros((40, 128, 128), np.float32)
+    r[0] = synth.normal_array(128 * 128, 3).reshape(128, 128)
+    rd, x = torch.from_numpy(r).to(DEV), torch.zeros(gg.n_cols, device=DEV)
+    cb = None if block is None else [block]
+    names = kernels_of(lambda: B.bsgd_back_project(gg, rd, x, col_blocks=cb))
+    assert ("bp_gather_kernel" in names) == gathers and ("bp_plain_kernel" in names) != gathers
+    ref = P.bp(og, r[0].reshape(-1).astype(np.float64)).reshape(128, -1)
+    sl = slice(None) if block is None else slice(32 * block, 32 * block + 32)
+    assert rel_l2(x.cpu().double().numpy().reshape(128, -1)[sl], ref[sl]) <= 4e-5
