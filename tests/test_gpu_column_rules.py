@@ -157,3 +157,21 @@ def test_sources_that_touch_the_volume_scatter(dso, block, gathers):
     ref = P.bp(og, r[0].reshape(-1).astype(np.float64)).reshape(128, -1)
     sl = slice(None) if block is None else slice(32 * block, 32 * block + 32)
     assert rel_l2(x.cpu().double().numpy().reshape(128, -1)[sl], ref[sl]) <= 4e-5
+
+
+@pytest.mark.parametrize("M", [1, 4, 7])
+def test_all_row_blocks_gather_in_view_order(M):
+    """All row blocks of a geometry give the sums of one block of all views, bit for
+    bit: the views are taken in order whichever blocks they are in."""
+    s = cone(64, 64, 30, 70, 70, 1.8, 200.0, 2.0, 1)
+    r = torch.from_numpy(synth.normal_array(30 * 70 * 70, 3).astype(np.float32)).to(DEV)
+    a, b = torch.zeros(64 ** 3, device=DEV), torch.zeros(64 ** 3, device=DEV)
+    B.bsgd_back_project(gpu_geom(s), r, a)
+    gg = gpu_geom(dict(s, M=M))
+    B.bsgd_back_project(gg, r, b)
+    assert torch.equal(a, b)
+    # some of the blocks, added one after another: the same sums in another order
+    c = torch.zeros_like(b)
+    for i in range(M):
+        B.bsgd_back_project(gg, r, c, row_blocks=[i], accumulate=True)
+    assert rel_l2(c.cpu().double().numpy(), a.cpu().double().numpy()) <= 1e-6
