@@ -129,7 +129,7 @@ extern "C" bsgd_status bsgd_back_project(const bsgd_geometry *g, const void *r, 
     int views = 0;
     for (int i : rows) views += (int)g->block_views[i].size();
     auto gathers = [&](const std::pair<int, int> &run) {
-        return column_bp_pays(g, g->plane_start[run.second] - g->plane_start[run.first], views);
+        return column_bp_pays(g, g->plane_start[run.first], g->plane_start[run.second], views);
     };
     const size_t W = std::any_of(runs.begin(), runs.end(), gathers) ? column_weights_len(g, std::min((int)rows.size(), 64)) : 0;
     if (W) pool_try_alloc((void **)&w, W * 4, st);

@@ -208,7 +208,7 @@ bsgd_status launch_count(const bsgd_geometry *g, const PlainLaunch &L,
 // from weights that it lays out row by row in `w` (column_weights_len floats; 0:
 // too many).
 bsgd_status column_tables(bsgd_geometry *g);
-bool column_bp_pays(const bsgd_geometry *g, int planes, int views);
+bool column_bp_pays(const bsgd_geometry *g, int z0, int z1, int views);
 size_t column_weights_len(const bsgd_geometry *g, int n_rb);
 // The same for images of a 2D kind: a thread per pixel, no weights.
 bool slice_bp_pays(const bsgd_geometry *g, int rows, int views);

@@ -266,7 +266,21 @@ static double gather_waste(const bsgd_geometry *g, int planes) {
     return (planes + 31) / 32 * 32.0 / planes * (d.dv * d.dso / d.dsd / d.dz);
 }
 
-// Whether the back projection of `views` views into `planes` planes gathers. A
+// Planes of [z0, z1) that a view's detector covers, on the mean over the depth of
+// the volume along the view.
+static double covered_planes(const bsgd_geometry *g, int z0, int z1) {
+    const bsgd_geometry_desc &d = g->desc;
+    const double depth = 0.5 * (d.nx * d.dx + d.ny * d.dy), mid = 0.5 * d.nz;
+    double sum = 0.0;
+    for (int k = 0; k < 8; ++k) {
+        const double s = ((k + 0.5) / 8.0 - 0.5) * depth;
+        const double reach = 0.5 * d.nv * d.dv * (d.dso - s) / d.dsd / d.dz;   // planes from the middle
+        sum += std::max(0.0, std::min(z1 - mid, reach) - std::max(z0 - mid, -reach));
+    }
+    return sum / 8.0;
+}
+
+// Whether the back projection of `views` views into planes [z0, z1) gathers. A
 // warp runs through all views of its column (0.43 us each, whatever the other
 // warps do), so small slabs seen from many views scatter instead: 64 x 64 x 32
 // from 360 views 151 us scattered, 164 gathered; 64^3 from 90 views 114 and 66
@@ -280,11 +294,17 @@ static double gather_waste(const bsgd_geometry *g, int planes) {
 // 60 views, source 5.5 voxels away [0.29] 731 / 462, 3.5 [0.62] 726 / 630, 2.5 [1.1]
 // 756 / 818; 256^3 from 45, 4 voxels [0.40] 3771 / 3285, 3 [0.69] 3799 / 4298; a
 // 32-plane slab of it, 9 voxels [0.77] 769 / 585, 5 [2.1] 804 / 1243.
-bool column_bp_pays(const bsgd_geometry *g, int planes, int views) {
+// A list costs a warp the same however few planes its rays then reach: slabs at the
+// end of a volume that the detector covers in part (covered planes in brackets): 512^2 x 32
+// from 45 views [5.1] 303 / 334, [7.8] 405 / 376, 128^2 x 32 from 360 [8.1] 398 / 441,
+// [9.6] 451 / 446, 256^2 x 32 from 360 [3.0] 417 / 641, [10.1] 989 / 877.
+bool column_bp_pays(const bsgd_geometry *g, int z0, int z1, int views) {
+    const int planes = z1 - z0;
     const int64_t plane = (int64_t)g->desc.nx * g->desc.ny, voxels = plane * planes;
     if (g->dg.nvp == 0 || planes <= 0 || voxels < (views <= 32 ? 64000 : 160000)) return false;
     const double pad = (double)g->desc.nu * 2.0 * g->dg.vpad;
-    return pad <= 0.64 * (double)(plane * g->desc.nz) && pad <= 1.2 * (double)voxels && gather_waste(g, planes) <= 1.7;
+    return pad <= 0.64 * (double)(plane * g->desc.nz) && pad <= 1.2 * (double)voxels && gather_waste(g, planes) <= 1.7 &&
+           covered_planes(g, z0, z1) >= 9.0;
 }
 
 static bsgd_status fill_tables(bsgd_geometry *g, bool slice) {

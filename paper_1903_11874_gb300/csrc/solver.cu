@@ -1155,7 +1155,7 @@ bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int 
     // iteration is the same, slower)
     int views = 0;
     for (int k = 0; k < n_rb; ++k) views += (int)g->block_views[row_ids[k]].size();
-    if (column_bp_pays(g, g->plane_start[j + 1] - g->plane_start[j], views)) {
+    if (column_bp_pays(g, g->plane_start[j], g->plane_start[j + 1], views)) {
         const size_t W = column_weights_len(g, std::min(n_rb, 64));
         if (W) pool_try_alloc((void **)&cw, W * 4, st);
     }

@@ -175,3 +175,15 @@ def test_all_row_blocks_gather_in_view_order(M):
     for i in range(M):
         B.bsgd_back_project(gg, r, c, row_blocks=[i], accumulate=True)
     assert rel_l2(c.cpu().double().numpy(), a.cpu().double().numpy()) <= 1e-6
+
+
+@pytest.mark.parametrize("pitch,block,gathers", [(1.2, 0, False), (1.2, 1, True), (1.6, 0, True)])
+def test_slabs_that_the_detector_hardly_covers_scatter(pitch, block, gathers):
+    """The rule on a slab's covered planes: the top slab of 128^3 scatters under a
+    detector that covers seven of its 32 planes."""
+    gg = gpu_geom(dict(cone(128, 128, 40, 128, 128, pitch, 250.0, 2.0, 4), M=2))
+    r, x = torch.ones(gg.n_rows, device=DEV), torch.zeros(gg.n_cols, device=DEV)
+    names = kernels_of(lambda: B.bsgd_back_project(gg, r, x, col_blocks=[block]))
+    assert ("bp_gather_kernel" in names) == gathers and ("bp_plain_kernel" in names) != gathers
+    names = kernels_of(lambda: B.bsgd_power_iteration(gg, block, 2))
+    assert ("bp_gather_kernel" in names) == gathers and ("bp_plain_kernel" in names) != gathers
