@@ -294,14 +294,16 @@ static double covered_planes(const bsgd_geometry *g, int z0, int z1) {
 // 60 views, source 5.5 voxels away [0.29] 731 / 462, 3.5 [0.62] 726 / 630, 2.5 [1.1]
 // 756 / 818; 256^3 from 45, 4 voxels [0.40] 3771 / 3285, 3 [0.69] 3799 / 4298; a
 // 32-plane slab of it, 9 voxels [0.77] 769 / 585, 5 [2.1] 804 / 1243.
-// A list costs a warp the same however few planes its rays then reach: slabs at the
-// end of a volume that the detector covers in part (covered planes in brackets): 512^2 x 32
+// A list costs a warp the same however few planes its rays then reach: 256^2 from 45
+// views, rows 0.5 / 0.8 voxel apart, 12 planes 248 / 307 and 184 / 193, 16 planes 313
+// / 309 and 218 / 195, 20 planes 376 / 312 and 265 / 196; slabs at the end of a
+// volume that the detector covers in part (covered planes in brackets): 512^2 x 32
 // from 45 views [5.1] 303 / 334, [7.8] 405 / 376, 128^2 x 32 from 360 [8.1] 398 / 441,
 // [9.6] 451 / 446, 256^2 x 32 from 360 [3.0] 417 / 641, [10.1] 989 / 877.
 bool column_bp_pays(const bsgd_geometry *g, int z0, int z1, int views) {
     const int planes = z1 - z0;
     const int64_t plane = (int64_t)g->desc.nx * g->desc.ny, voxels = plane * planes;
-    if (g->dg.nvp == 0 || planes <= 0 || voxels < (views <= 32 ? 64000 : 160000)) return false;
+    if (g->dg.nvp == 0 || planes < 16 || voxels < (views <= 32 ? 64000 : 160000)) return false;
     const double pad = (double)g->desc.nu * 2.0 * g->dg.vpad;
     return pad <= 0.64 * (double)(plane * g->desc.nz) && pad <= 1.2 * (double)voxels && gather_waste(g, planes) <= 1.7 &&
            covered_planes(g, z0, z1) >= 9.0;

@@ -187,3 +187,12 @@ def test_slabs_that_the_detector_hardly_covers_scatter(pitch, block, gathers):
     assert ("bp_gather_kernel" in names) == gathers and ("bp_plain_kernel" in names) != gathers
     names = kernels_of(lambda: B.bsgd_power_iteration(gg, block, 2))
     assert ("bp_gather_kernel" in names) == gathers and ("bp_plain_kernel" in names) != gathers
+
+
+@pytest.mark.parametrize("planes,gathers", [(12, False), (16, True)])
+def test_thin_slabs_of_fine_rows_scatter(planes, gathers):
+    """The rule on a slab's planes holds for rows close together, too."""
+    gg = gpu_geom(cone(128, planes, 40, 128, 128, 1.0, 250.0, 2.0, 1))
+    r, x = torch.ones(gg.n_rows, device=DEV), torch.zeros(gg.n_cols, device=DEV)
+    names = kernels_of(lambda: B.bsgd_back_project(gg, r, x))
+    assert ("bp_gather_kernel" in names) == gathers and ("bp_plain_kernel" in names) != gathers
