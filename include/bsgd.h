@@ -459,7 +459,10 @@ bsgd_status bsgd_state_profile(bsgd_state *s, int enable);
  * n_cells as in bsgd_solve_params). The memory of every (block, cell) is kept,
  * so switching from BSGD-IM to whole views continues the same SAG estimate.
  * Iterations already launched are unaffected. May compute the geometry's
- * tables for the new cell count (synchronises `stream` then).
+ * tables for the new cell count (synchronises `stream` then). A cone-beam state
+ * of one column block per iteration that gathers with whole views scatters with
+ * cells: it then exchanges the memory of the two forms (in stream order; without
+ * room for the other's it keeps its own).
  * Errors: INVALID_ARG (residual pairs with more than one pair per iteration,
  * bad mode or cell count).
  */

@@ -941,6 +941,7 @@ struct bsgd_state {
     void *xT = nullptr;         // y-fastest copy of x (volumes only)
     float *gT = nullptr;        // y-fastest part of g (volumes only)
     float *w = nullptr;         // column form: weights of an iteration's BP (then no gT)
+    bool column = false;        // the column form is taken where it pays
     float *grad = nullptr;
     double *S = nullptr, *cw = nullptr, *d_mu = nullptr;
     Work *work = nullptr;
@@ -1364,6 +1365,7 @@ static bsgd_status create_form(const bsgd_geometry *g, const bsgd_solve_params *
     s->st = (bsgd_dtype)p->storage;
     s->fused = s->kN == 1;
     s->n_cells = p->cells == BSGD_CELLS_NONE ? 1 : p->n_cells;
+    s->column = column;
     if (s->P > kMaxPairs) {
         free_state(s);
         return fail(BSGD_ERR_INVALID_ARG, "more than 64 pairs per iteration");
@@ -1961,6 +1963,33 @@ extern "C" bsgd_status bsgd_state_profile(bsgd_state *s, int enable) {
     return BSGD_OK;
 }
 
+// The form of the BP that pays with the state's cells (column_solve_len), taken
+// when they change: g is whole in the column form and has a y-fastest part in the
+// other. Without room for the other form's memory the state keeps the one it has.
+static bsgd_status follow_cells(bsgd_state *s, cudaStream_t st) {
+    const bsgd_geometry *g = s->g;
+    const size_t W = s->column ? column_solve_len(g, s->kM, s->kN, s->p.cells != BSGD_CELLS_NONE) : 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((W != 0) == (s->w != nullptr) || g->desc.nz == 1 ||
+        cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return BSGD_OK;
+    float *now = nullptr;
+    const size_t bytes = W ? W * 4 : (size_t)g->n_cols() * 4;
+    if (!pool_try_alloc((void **)&now, bytes, st)) return BSGD_OK;
+    bsgd_status e = cudaMemsetAsync(now, 0, bytes, st) == cudaSuccess ? BSGD_OK : fail(BSGD_ERR_CUDA, "cudaMemsetAsync failed");
+    if (!e && W) e = plain_add_transposed(g, s->gT, s->grad, 0, g->N, st);
+    if (e) {
+        pool_free(now, st);
+        return e;
+    }
+    pool_free(W ? s->gT : s->w, st);
+    s->gT = W ? nullptr : now;
+    s->w = W ? now : nullptr;
+    s->dev.gT = s->gT;
+    s->dev.w = s->w;
+    return BSGD_OK;
+}
+
 extern "C" bsgd_status bsgd_state_set_sampling(bsgd_state *s, int pair_sampling, int cells,
                                                int n_cells, void *stream) {
     if (!s) return fail(BSGD_ERR_INVALID_ARG, "state is NULL");
@@ -1989,7 +2018,7 @@ extern "C" bsgd_status bsgd_state_set_sampling(bsgd_state *s, int pair_sampling,
     pair_updates_kernel<<<(g->M * g->N + 127) / 128, 128, 0, (cudaStream_t)stream>>>(
         g->dg, counts, nc, s->pair_upd);
     BSGD_CUDA(cudaGetLastError());
-    return BSGD_OK;
+    return follow_cells(s, (cudaStream_t)stream);
 }
 
 extern "C" bsgd_status bsgd_state_set_split(bsgd_state *s, int split) {

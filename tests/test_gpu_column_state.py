@@ -1,5 +1,6 @@
 """Solver states around the gathering back projection: checkpoints between a
-state that gathers and one that scatters, and the memory that a state needs."""
+state that gathers and one that scatters, the memory that a state needs, and a
+change of the sampling mode."""
 import os
 import struct
 import subprocess
@@ -13,6 +14,7 @@ from helpers import gpu_geom, oracle_geom, rel_l2
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+from oracle import bsgd as OB  # noqa: E402
 from oracle import projector as P  # noqa: E402
 from paper_1903_11874_gb300 import binding as B  # noqa: E402
 from paper_1903_11874_gb300 import synth  # noqa: E402
@@ -142,3 +144,41 @@ def test_little_memory_scatters():
     res = subprocess.run([sys.executable, "-c", LITTLE_MEMORY], cwd=os.path.dirname(here), env=env,
                          capture_output=True, text=True, timeout=300)
     assert "MADE" in res.stdout, res.stderr[-2000:]
+
+
+def kernels_of(f):
+    """Names of the kernels that a call launches."""
+    for _ in range(3):   # (a process's first profile comes back empty)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            f()
+            torch.cuda.synchronize()
+        names = " ".join(e.key for e in prof.key_averages())
+        if "kernel" in names:
+            break
+    return names
+
+
+@pytest.mark.parametrize("first", [B.CELLS_NONE, B.CELLS_UNIFORM])
+def test_sampling_mode_carries_the_form(one_block, first):
+    """A one-block state gathers while it draws whole views and scatters while it
+    draws cells, whatever it was created with; its image after changes of the mode
+    both ways is the oracle's of the same draws (the solver tests' bound)."""
+    gg, y = one_block
+    s = solve_geometry(1)
+    og = oracle_geom(s)
+    st = one_block_state(one_block, first)
+    x = torch.zeros(gg.n_cols, device=DEV)
+    modes = [B.CELLS_NONE, B.CELLS_UNIFORM, B.CELLS_NONE, B.CELLS_UNIFORM]
+    for m in modes:
+        st.set_sampling(B.PAIRS_UNIFORM, m, 1 if m == B.CELLS_NONE else 4)
+        st.block_step(x, 2)
+    sels = []
+    for t in st.read_trace(8):
+        c = t[3:3 + gg.n_views].astype(np.int64)
+        sels.append(OB.Selection([(int(t[1]), int(t[2]))], [None if c[0] < 0 else c]))
+    po = OB.Params(1, 2, 1.0, 0.5, 2e-5, seed=5, cells="uniform", n_cells=4)
+    ost = OB.bsgd(og, y.cpu().double().numpy(), po, 8, replay=sels)
+    assert rel_l2(x.cpu().double().numpy(), ost.x) <= 1e-5
+    for m, gathers in ((B.CELLS_NONE, True), (B.CELLS_UNIFORM, False)):
+        st.set_sampling(B.PAIRS_UNIFORM, m, 1 if m == B.CELLS_NONE else 4)
+        assert ("solve_gather_kernel" in kernels_of(lambda: st.block_step(x, 2))) == gathers
