@@ -123,16 +123,7 @@ struct bsgd_geometry {
     int64_t zlen = 0;
     int device = 0;
     // device copies
-    bsgd::ViewRay *d_rays = nullptr;
-    bsgd::Band *d_bands = nullptr;
-    int *d_block_views = nullptr;
-    int *d_block_nviews = nullptr;
-    int *d_plane_start = nullptr;
-    int *d_view_block = nullptr;
-    unsigned char *d_view_yfast = nullptr;
-    int64_t *d_zoff = nullptr;
-    bsgd::ColRay *d_cray = nullptr;
-    float2 *d_slice = nullptr;
+    char *d_tables = nullptr;   // all tables that dg points to
     bsgd::DeviceGeom dg{};
     // Filled on first use by a solver state and kept for the geometry's life
     // (index: number of detector cells 1, 2 or 4): exact voxel-ray update
@@ -203,11 +194,13 @@ bsgd_status plain_add_transposed(const bsgd_geometry *g, const float *gT, float 
                                  cudaStream_t st);
 bsgd_status launch_count(const bsgd_geometry *g, const PlainLaunch &L,
                          unsigned long long *d_count, cudaStream_t st);
-// Column form of the cone beam (column.cu). column_tables fills the geometry's
-// tables where the form applies; launch_bp_column back-projects by gathering,
+// Column form of the cone beam (column.cu). column_plan sets the form's constants
+// and returns the bytes of its tables (0: it does not apply), which column_tables
+// fills; launch_bp_column back-projects by gathering,
 // from weights that it lays out row by row in `w` (column_weights_len floats; 0:
 // too many).
-bsgd_status column_tables(bsgd_geometry *g);
+size_t column_plan(bsgd_geometry *g);
+bsgd_status column_tables(bsgd_geometry *g, void *tables);
 bool column_bp_pays(const bsgd_geometry *g, int z0, int z1, int views);
 size_t column_weights_len(const bsgd_geometry *g, int n_rb);
 // The same for images of a 2D kind: a thread per pixel, no weights.

@@ -309,28 +309,31 @@ bool column_bp_pays(const bsgd_geometry *g, int z0, int z1, int views) {
            covered_planes(g, z0, z1) >= 9.0;
 }
 
-static bsgd_status fill_tables(bsgd_geometry *g, bool slice) {
+// Lines of a 2D kind (arrays, DeviceGeom::sx) or of a cone (records).
+bsgd_status column_tables(bsgd_geometry *g, void *tables) {
     DeviceGeom &dg = g->dg;
     const int64_t n = (int64_t)g->desc.n_views * g->desc.nu;
-    if (slice) BSGD_CUDA(cudaMalloc((void **)&g->d_slice, 28 * (size_t)n));
-    else BSGD_CUDA(cudaMalloc((void **)&g->d_cray, sizeof(ColRay) * (size_t)n));
+    const bool slice = g->desc.kind != BSGD_CONE3D;
+    ColRay *cray = slice ? nullptr : (ColRay *)tables;
+    float2 *lines = slice ? (float2 *)tables : nullptr;
     const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 152 * 16));
-    column_tables_kernel<<<gb, 128>>>(dg, g->d_cray, g->d_slice);
+    column_tables_kernel<<<gb, 128>>>(dg, cray, lines);
     BSGD_CUDA(cudaGetLastError());
     BSGD_CUDA(cudaStreamSynchronize(0));
-    dg.cray = g->d_cray;
+    dg.cray = cray;
     if (slice) {
-        dg.sx = g->d_slice;
-        dg.sy = g->d_slice + n;
-        dg.si = g->d_slice + 2 * n;
-        dg.slen = reinterpret_cast<float *>(g->d_slice + 3 * n);
+        dg.sx = lines;
+        dg.sy = lines + n;
+        dg.si = lines + 2 * n;
+        dg.slen = reinterpret_cast<float *>(lines + 3 * n);
     }
     return BSGD_OK;
 }
 
-bsgd_status column_tables(bsgd_geometry *g) {
+size_t column_plan(bsgd_geometry *g) {
     const bsgd_geometry_desc &d = g->desc;
     DeviceGeom &dg = g->dg;
+    const size_t rays = (size_t)d.n_views * d.nu;
     // a line's ends, and the products of the lengths that give a shadow, round to
     // 2^-24 of the ray's length each: eight of these in detector columns (with
     // 0.01 alone, a fan from 1e6 voxels away lost 3e-4 of the sum)
@@ -339,22 +342,22 @@ bsgd_status column_tables(bsgd_geometry *g) {
     dg.umargin = (float)(0.01 + rounding);
     if (d.kind != BSGD_CONE3D) {
         dg.tc = d.kind == BSGD_PAR2D ? 0.5f : (float)(d.dso / d.dsd);
-        return fill_tables(g, true);
+        return 28 * rays;
     }
-    if (d.nz < 2 || d.nv < 2) return BSGD_OK;
+    if (d.nz < 2 || d.nv < 2) return 0;
     // FP32 holds the place along a ray where it crosses a plane to 2^-24 of its
     // length: up to a hundredth of a voxel, which a row of rays that lies along a
     // face loses (1e-4 of its sum at 6e5 voxels, where the walk loses 2e-6); and
     // rays that round to half a column or more could meet voxels outside the bands,
     // where no weights are laid out
-    if (std::ldexp(length / std::min(d.dx, d.dy), -24) > 0.01 || rounding > 1.0) return BSGD_OK;
+    if (std::ldexp(length / std::min(d.dx, d.dy), -24) > 0.01 || rounding > 1.0) return 0;
     // rows are found by an addition that holds them in 22 bits, and to 0.01 by FP32
     // from the detector's middle
     const double near = d.dso - 0.5 * std::hypot(d.nx * d.dx, d.ny * d.dy);
-    if (d.nv > (1 << 14) || d.dz * d.dsd / (near * d.dv) > 1e3) return BSGD_OK;
+    if (d.nv > (1 << 14) || d.dz * d.dsd / (near * d.dv) > 1e3) return 0;
     // a ray rises less than a voxel while it crosses a column
     const double rise = 0.5 * (d.nv - 1) * d.dv / d.dz / d.dsd;   // voxels per mm along the axis
-    if (std::sqrt(2.0) * std::max(d.dx, d.dy) * rise > 0.95) return BSGD_OK;
+    if (std::sqrt(2.0) * std::max(d.dx, d.dy) * rise > 0.95) return 0;
     dg.tc = (float)(d.dso / d.dsd);
     dg.zs = g->rays[0].p0[2];
     dg.vstep = g->rays[0].cv[2];
@@ -365,7 +368,7 @@ bsgd_status column_tables(bsgd_geometry *g) {
     dg.vslack = (float)(32.0 * change * 1.01);
     dg.vpad = (int)std::ceil(33.0 * rows + (2.0 * d.nz + 32.0) * change) + 8;
     dg.nvp = (d.nv + 2 * dg.vpad + 7) / 8 * 8;
-    return fill_tables(g, false);
+    return sizeof(ColRay) * rays;
 }
 
 size_t column_weights_len(const bsgd_geometry *g, int n_rb) {

@@ -196,3 +196,18 @@ def test_thin_slabs_of_fine_rows_scatter(planes, gathers):
     r, x = torch.ones(gg.n_rows, device=DEV), torch.zeros(gg.n_cols, device=DEV)
     names = kernels_of(lambda: B.bsgd_back_project(gg, r, x))
     assert ("bp_gather_kernel" in names) == gathers and ("bp_plain_kernel" in names) != gathers
+
+
+@pytest.mark.parametrize("s", [cone(64, 64, 30, 70, 70, 1.8, 200.0, 2.0, 4), fan(70, 60, 97, 2, np.arange(60) % 2)])
+def test_geometry_is_one_allocation(s):
+    """All tables of a geometry, the gather's lines among them, are one block of
+    device memory."""
+    gpu_geom(s)
+    for _ in range(3):   # (a process's first profile comes back empty)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            gpu_geom(s)
+            torch.cuda.synchronize()
+        calls = {e.key: e.count for e in prof.key_averages()}
+        if "cudaMalloc" in calls:
+            break
+    assert calls["cudaMalloc"] == 1
