@@ -366,7 +366,9 @@ size_t column_plan(bsgd_geometry *g) {
     const double rows = d.dz * d.dsd / (near * d.dv);
     const double change = rows * std::sqrt(2.0) * std::max(d.dx, d.dy) / near;   // rows per voxel of height
     dg.vslack = (float)(32.0 * change * 1.01);
-    dg.vpad = (int)std::ceil(33.0 * rows + (2.0 * d.nz + 32.0) * change) + 8;
+    const double pad = std::ceil(33.0 * rows + (2.0 * d.nz + 32.0) * change) + 8.0;
+    if (pad > 1e6) return 0;   // a source in the volume's corner: past any use, and past int
+    dg.vpad = (int)pad;
     dg.nvp = (d.nv + 2 * dg.vpad + 7) / 8 * 8;
     return sizeof(ColRay) * rays;
 }

@@ -211,3 +211,21 @@ def test_geometry_is_one_allocation(s):
         if "cudaMalloc" in calls:
             break
     assert calls["cudaMalloc"] == 1
+
+
+def test_source_in_the_corner_scatters():
+    """A source 0.0035 voxel from the corner of a tall volume, where the padding of
+    the weights would not fit an int: the back projection takes the walk.
+
+    Bound: that of the plain gather's tests at the rounding of heights up to 1500
+    voxels (6.1e-5, eight times theirs), against the oracle."""
+    s = cone(8, 3000, 4, 9, 4, 3.3, 8 / np.sqrt(2.0) + 0.0035, 2.0, 1)
+    near = s["dso"] - 8 / np.sqrt(2.0)
+    rows = s["dsd"] / (near * s["dv"])
+    assert rows < 1e3 and s["dv"] / 2.0 <= 1.7 and (2 * 3000 + 32) * rows * np.sqrt(2.0) / near > 2 ** 31
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = synth.normal_array(og.n_rows, 3).astype(np.float32)
+    rd, x = torch.from_numpy(r).to(DEV), torch.zeros(og.n_cols, device=DEV)
+    names = kernels_of(lambda: B.bsgd_back_project(gg, rd, x))
+    assert "bp_gather_kernel" not in names and "bp_plain_kernel" in names
+    assert rel_l2(x.cpu().double().numpy(), P.bp(og, r.astype(np.float64)).reshape(-1)) <= 3.2e-4
