@@ -198,11 +198,13 @@ bsgd_status launch_count(const bsgd_geometry *g, const PlainLaunch &L,
 // and returns the bytes of its tables (0: it does not apply), which column_tables
 // fills; launch_bp_column back-projects by gathering,
 // from weights that it lays out row by row in `w` (column_weights_len floats; 0:
-// too many).
+// too many), `per` row blocks at a time (at most 64): column_blocks_within of them
+// have weights of at most so many floats.
 size_t column_plan(bsgd_geometry *g);
 bsgd_status column_tables(bsgd_geometry *g, void *tables);
 bool column_bp_pays(const bsgd_geometry *g, int z0, int z1, int views);
 size_t column_weights_len(const bsgd_geometry *g, int n_rb);
+int column_blocks_within(const bsgd_geometry *g, int n_rb, size_t floats);
 // The same for images of a 2D kind: a thread per pixel, no weights.
 bool slice_bp_pays(const bsgd_geometry *g, int rows, int views);
 bsgd_status launch_bp_slice(const bsgd_geometry *g, const PlainLaunch &L, const void *r, bsgd_dtype rt,
@@ -210,7 +212,7 @@ bsgd_status launch_bp_slice(const bsgd_geometry *g, const PlainLaunch &L, const 
 size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells);
 bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const void *r,
                              bsgd_dtype rt, float *x, float scale, int accumulate, float *w,
-                             cudaStream_t st);
+                             cudaStream_t st, int per = 64);
 // Clear the rows of every view of the listed row blocks.
 bsgd_status zero_rows(const bsgd_geometry *g, const int *row_ids, int n_rb, void *y,
                       bsgd_dtype yt, cudaStream_t st);

@@ -379,6 +379,12 @@ size_t column_weights_len(const bsgd_geometry *g, int n_rb) {
     return n < (1ull << 32) ? n : 0;
 }
 
+int column_blocks_within(const bsgd_geometry *g, int n_rb, size_t floats) {
+    int n = std::min(n_rb, 64);
+    while (n > 0 && (column_weights_len(g, n) == 0 || column_weights_len(g, n) > floats)) --n;
+    return n;
+}
+
 static dim3 gather_grid(const bsgd_geometry *g, int planes, int z) {
     const int across = (g->desc.nx + kGatherAcross - 1) / kGatherAcross, rows = (g->desc.ny + kGatherRows - 1) / kGatherRows;
     return dim3((unsigned)(across * rows), (planes + 32 * kGatherChunks - 1) / (32 * kGatherChunks), z);
@@ -386,12 +392,12 @@ static dim3 gather_grid(const bsgd_geometry *g, int planes, int z) {
 
 bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const void *r,
                              bsgd_dtype rt, float *x, float scale, int accumulate, float *w,
-                             cudaStream_t st) {
+                             cudaStream_t st, int per) {
     const int z0 = g->plane_start[L.j0], z1 = g->plane_start[L.j1];
     const dim3 grid = gather_grid(g, z1 - z0, 1);
-    for (int k = 0; k < L.n_rb; k += 64) {
+    for (int k = 0; k < L.n_rb; k += per) {
         RowSel R{};
-        R.n = std::min(64, L.n_rb - k);
+        R.n = std::min(per, L.n_rb - k);
         for (int t = 0; t < R.n; ++t) R.ids[t] = L.row_ids[k + t];
         const dim3 wg((unsigned)((g->desc.nu + 31) / 32 * ((g->dg.nvp + 31) / 32)), gather_slots(g->dg, R));
         if (rt == BSGD_F32) column_weights_kernel<float><<<wg, 256, 0, st>>>(g->dg, R, L.j0, L.j1, (const float *)r, scale, w);

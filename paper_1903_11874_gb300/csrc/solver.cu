@@ -1126,9 +1126,10 @@ bsgd_status norm_table(const bsgd_geometry *g, const void *r, bsgd_dtype t, doub
     return BSGD_OK;
 }
 
-// lambda ~ ||A_rows^J||^2 by power iteration (see bsgd.h).
+// lambda ~ ||A_rows^J||^2 by power iteration (see bsgd.h). most: floats that the
+// weights of its gathering BP may take.
 bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int *row_ids, int n_rb,
-                            double *lambda, cudaStream_t st) {
+                            double *lambda, cudaStream_t st, size_t most = SIZE_MAX) {
     const int64_t b0 = (int64_t)g->plane_start[j] * g->dg.plane_stride;
     const int64_t b1 = (int64_t)g->plane_start[j + 1] * g->dg.plane_stride;
     const int64_t n = g->n_cols(), m = g->n_rows();
@@ -1154,11 +1155,11 @@ bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int 
     // the column form's weights, or y-fastest copies for the views whose rays run
     // along x: of the BP accumulator, and of v (optional: without them the
     // iteration is the same, slower)
-    int views = 0;
+    int views = 0, per = 0;
     for (int k = 0; k < n_rb; ++k) views += (int)g->block_views[row_ids[k]].size();
     if (column_bp_pays(g, g->plane_start[j], g->plane_start[j + 1], views)) {
-        const size_t W = column_weights_len(g, std::min(n_rb, 64));
-        if (W) pool_try_alloc((void **)&cw, W * 4, st);
+        per = column_blocks_within(g, n_rb, most);
+        if (per) pool_try_alloc((void **)&cw, column_weights_len(g, per) * 4, st);
     }
     if (plain_wants_transpose(g, row_ids, n_rb)) {
         pool_try_alloc((void **)&vT, n * 4, st);
@@ -1170,7 +1171,7 @@ bsgd_status power_iteration(const bsgd_geometry *g, int j, int iters, const int 
         BSGD_CUDA(cudaMemsetAsync(y, 0, m * 4, st));
         if (vT) BSGD_TRY(plain_transpose(g, v32, BSGD_F32, vT, j, j + 1, st));
         BSGD_TRY(launch_fp_plain(g, L, v32, BSGD_F32, y, BSGD_F32, 1, st, vT));
-        if (cw) return launch_bp_column(g, L, y, BSGD_F32, w, 1.0f, 0, cw, st);
+        if (cw) return launch_bp_column(g, L, y, BSGD_F32, w, 1.0f, 0, cw, st, per);
         if (slice_bp_pays(g, g->plane_start[j + 1] - g->plane_start[j], views))
             return launch_bp_slice(g, L, y, BSGD_F32, w, 1.0f, 0, st);
         if (wT) BSGD_CUDA(cudaMemsetAsync(wT + b0, 0, (b1 - b0) * 4, st));
@@ -1446,15 +1447,18 @@ static bsgd_status create_form(const bsgd_geometry *g, const bsgd_solve_params *
                     cached = true;
                 }
             }
+            // a served request's memory is counted with the y-fastest accumulator
+            // that the weights replace: they take no more
+            const size_t most = column ? SIZE_MAX : (size_t)C;
             for (int j = 0; j < N && !cached; ++j) {
                 if (p->step_rule == BSGD_STEP_STRIP) {
                     double lam = 0.0;
-                    BSGD_TRY(power_iteration(g, j, p->power_iters, nullptr, 0, &lam, st));
+                    BSGD_TRY(power_iteration(g, j, p->power_iters, nullptr, 0, &lam, st, most));
                     lmax = std::max(lmax, lam);
                 } else {
                     for (int i = 0; i < M; ++i) {
                         double lam = 0.0;
-                        BSGD_TRY(power_iteration(g, j, p->power_iters, &i, 1, &lam, st));
+                        BSGD_TRY(power_iteration(g, j, p->power_iters, &i, 1, &lam, st, most));
                         lmax = std::max(lmax, lam);
                     }
                 }

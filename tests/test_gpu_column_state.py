@@ -182,3 +182,29 @@ def test_sampling_mode_carries_the_form(one_block, first):
     for m, gathers in ((B.CELLS_NONE, True), (B.CELLS_UNIFORM, False)):
         st.set_sampling(B.PAIRS_UNIFORM, m, 1 if m == B.CELLS_NONE else 4)
         assert ("solve_gather_kernel" in kernels_of(lambda: st.block_step(x, 2))) == gathers
+
+
+def test_served_set_up_keeps_to_its_bytes():
+    """The power iteration of a served request takes weights of at most an image's
+    floats (the y-fastest accumulator that its bytes are counted without): one row
+    block of four at a time here. Its step is the plain state's (FP32 sums in
+    another order)."""
+    geo = dict(kind="cone3d", nx=96, ny=96, nz=64, dx=1.0, dy=1.0, dz=1.0, n_views=96, nu=96, nv=96, du=1.7,
+               dv=1.7, dso=250.0, dsd=500.0)
+    prm = B.SolveParams(alpha=0.25, gamma=0.5, step_rule=B.STEP_STRIP, power_iters=3, rho=0.5, seed=5, epochs=1)
+    gg = B.Geometry(M=4, N=2, **geo)
+    y = np.ones(gg.n_rows, dtype=np.float32)
+    srv = B.Server(budget_bytes=4 << 30, max_slots=2)
+    try:
+        for _ in range(3):   # (a process's first profile comes back empty)
+            with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+                _x, rep = srv.wait(srv.submit(geo, 4, 2, prm, y))
+                torch.cuda.synchronize()
+            launches = sum(e.count for e in prof.key_averages() if "bp_gather_kernel" in e.key)
+            if launches:
+                break
+    finally:
+        srv.close()
+    assert launches == 2 * 3 * 4   # blocks x iterations x passes
+    st = B.State(gg, prm, torch.from_numpy(y).to(DEV))
+    assert abs(rep["mu"] / st.query()["mu"] - 1.0) <= 1e-5
