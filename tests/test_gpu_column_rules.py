@@ -229,3 +229,19 @@ def test_source_in_the_corner_scatters():
     names = kernels_of(lambda: B.bsgd_back_project(gg, rd, x))
     assert "bp_gather_kernel" not in names and "bp_plain_kernel" in names
     assert rel_l2(x.cpu().double().numpy(), P.bp(og, r.astype(np.float64)).reshape(-1)) <= 3.2e-4
+
+
+def test_more_row_blocks_than_a_launch_takes():
+    """66 row blocks of a cone (64 at a time): the second launch adds to the first's
+    image. Unequal voxel sides and angles given by the caller. The bounds are those
+    of the plain gather's tests."""
+    s = dict(kind="cone3d", nx=64, ny=60, nz=48, dx=1.0, dy=1.2, dz=0.9, n_views=66, nu=60, nv=50, du=2.3, dv=1.7,
+             dso=200.0, dsd=400.0, M=66, N=1, angles=np.sort(synth.uniform_array(66, 7)) * 6.28)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = synth.normal_array(og.n_rows, 3).astype(np.float32)
+    rd, x = torch.from_numpy(r).to(DEV), torch.full((og.n_cols,), 5.0, device=DEV)
+    assert kernels_of(lambda: B.bsgd_back_project(gg, rd, x)).count("bp_gather_kernel") == 1
+    assert rel_l2(x.cpu().double().numpy(), P.bp(og, r.astype(np.float64)).reshape(-1)) <= 4e-5
+    again = torch.zeros_like(x)
+    B.bsgd_back_project(gg, rd, again)
+    assert torch.equal(again, x)

@@ -208,3 +208,83 @@ def test_served_set_up_keeps_to_its_bytes():
     assert launches == 2 * 3 * 4   # blocks x iterations x passes
     st = B.State(gg, prm, torch.from_numpy(y).to(DEV))
     assert abs(rep["mu"] / st.query()["mu"] - 1.0) <= 1e-5
+
+
+KINDS = {"none": B.CELLS_NONE, "geometric": B.CELLS_GEOMETRIC, "uniform": B.CELLS_UNIFORM}
+
+
+@pytest.fixture(scope="module")
+def two_blocks():
+    s = solve_geometry(2)
+    og = oracle_geom(s)
+    return og, gpu_geom(s), scan(og, s)
+
+
+def check_against_oracle(st, x, ost, tol):
+    assert rel_l2(x.float().cpu().double().numpy(), ost.x) <= tol
+    rn = ost.residual_norm()
+    assert abs(st.query()["residual_norm"] - rn) <= tol * rn
+
+
+@pytest.mark.parametrize("kN,cells,storage", [(1, "none", "f32"), (2, "none", "f32"), (2, "uniform", "f32"),
+                                              (2, "geometric", "bf16")])
+def test_separate_passes(one_block, two_blocks, kN, cells, storage):
+    """FP, residual and BP apart: the weights are the residual's change on the
+    block's band (zero off the drawn cell), turned row by row, and the snapshot
+    follows. The solver tests' bounds."""
+    if kN == 1:
+        og, gg, y = oracle_geom(solve_geometry(1)), one_block[0], one_block[1].cpu().numpy()
+    else:
+        og, gg, y = two_blocks
+    n_cells = 1 if cells == "none" else 4
+    prm = B.SolveParams(alpha=1 / gg.M, gamma=kN / 2, step_rule=B.STEP_FIXED, mu=2e-5, seed=5, cells=KINDS[cells],
+                        n_cells=n_cells, storage=B.F32 if storage == "f32" else B.BF16)
+    st = B.State(gg, prm, torch.from_numpy(y).to(DEV))
+    x = torch.zeros(gg.n_cols, device=DEV, dtype=torch.float32 if storage == "f32" else torch.bfloat16)
+    st.block_step(x, 1)      # the passes alternate: both leave the same memory
+    st.set_split(True)
+    st.block_step(x, 3)
+    ost = OB.bsgd(og, y.astype(np.float64), OB.Params(gg.M, 2, 1 / gg.M, kN / 2, 2e-5, seed=5, cells=cells,
+                                                      n_cells=n_cells), 4)
+    check_against_oracle(st, x, ost, 1e-5 if storage == "f32" else 1e-2)
+    assert "column_change_kernel" in kernels_of(lambda: st.block_step(x, 1))
+
+
+def test_replayed_pairs(two_blocks):
+    """A replayed trace of several blocks takes the separate passes; it gives the
+    image of the draws it replays."""
+    og, gg, y = two_blocks
+    yd = torch.from_numpy(y).to(DEV)
+    kw = dict(alpha=0.5, gamma=1.0, step_rule=B.STEP_FIXED, mu=2e-5)
+    a, b = B.State(gg, B.SolveParams(seed=5, **kw), yd), B.State(gg, B.SolveParams(seed=6, **kw), yd)
+    xa, xb = torch.zeros(gg.n_cols, device=DEV), torch.zeros(gg.n_cols, device=DEV)
+    a.block_step(xa, 4)
+    trace = a.read_trace(4)
+    b.set_replay(trace)
+    b.block_step(xb, 4)
+    sels = [OB.Selection([(int(t[1]), int(t[2])), (int(t[3]), int(t[4]))], [None, None]) for t in trace]
+    ost = OB.bsgd(og, y.astype(np.float64), OB.Params(2, 2, 0.5, 1.0, 2e-5, seed=6), 4, replay=sels)
+    check_against_oracle(b, xb, ost, 1e-5)
+
+
+@pytest.mark.parametrize("cells", ["none", "uniform"])
+def test_sharded_steps(two_blocks, cells):
+    """One process that owns both blocks, and two that own one each (their parts of
+    the sum added here), with a gathering BP."""
+    og, gg, y = two_blocks
+    yd = torch.from_numpy(y).to(DEV)
+    n_cells = 1 if cells == "none" else 4
+    prm = B.SolveParams(alpha=0.5, gamma=1.0, step_rule=B.STEP_FIXED, mu=2e-5, seed=5, cells=KINDS[cells],
+                        n_cells=n_cells)
+    ost = OB.bsgd(og, y.astype(np.float64), OB.Params(2, 2, 0.5, 1.0, 2e-5, seed=5, cells=cells, n_cells=n_cells), 4)
+    for owners in ([[0, 1]], [[0], [1]]):
+        states = [B.State(gg, prm, yd) for _ in owners]
+        xs = [torch.zeros(gg.n_cols, device=DEV) for _ in owners]
+        parts = [torch.zeros(st.set_shard(own), device=DEV) for st, own in zip(states, owners)]
+        for _ in range(4):
+            for st, x, e in zip(states, xs, parts):
+                st.shard_begin(x, e)
+            total = sum(parts[1:], parts[0].clone())
+            for st, x in zip(states, xs):
+                st.shard_end(x, total)
+        check_against_oracle(states[0], sum(xs[1:], xs[0].clone()), ost, 1e-5)
