@@ -848,7 +848,8 @@ def paper_scale_leg(B, torch, dev, cases, warm=2, iters=10):
                 "alpha=0.2, gamma=0.5, geometric detector quadrants (Algorithm 2)" if im
                 else "alpha=1/5, gamma=2/8"),
             "ms_per_iteration": round(ms, 3),
-            "fused_ms_per_iteration": round(prof["fpbp"]["ms"] / iters, 3),
+            "pass": "fused" if prof["fpbp"]["launches"] else "fp, residual, bp",
+            "passes_ms_per_iteration": round(sum(prof[k]["ms"] for k in ("fpbp", "fp", "residual", "bp")) / iters, 3),
             "split_ms_per_iteration": round(ms_split, 3),
             "fp_ms_per_iteration": round(prs["fp"]["ms"] / iters, 3),
             "residual_ms_per_iteration": round(prs["residual"]["ms"] / iters, 3),

@@ -441,7 +441,8 @@ typedef enum {
     BSGD_STAGE_UPDATE = 4,   /* x_J += mu g_J                                 */
     BSGD_STAGE_TV = 5,       /* TV proximal step (BSGD-TV)                    */
     BSGD_STAGE_FPBP = 6,     /* FP, residual and BP in one pass (1 to 4 column
-                                blocks per iteration), counted once: one
+                                blocks per iteration; bsgd_state_set_split says
+                                when they are separate), counted once: one
                                 kernel, or the FP with the residual and the
                                 gathering BP                                  */
     BSGD_N_STAGES = 7
@@ -470,9 +471,11 @@ bsgd_status bsgd_state_set_sampling(bsgd_state *s, int pair_sampling, int cells,
                                     void *stream);
 
 /* split = 1: run FP, the residual (with several column blocks per iteration)
- * and BP as separate kernels (to time them apart); default 0: one fused kernel
+ * and BP as separate kernels (to time them apart); default 0: one fused pass
  * when 1 to 4 column blocks are drawn per iteration (with 2 to 4: uniform
- * pair draws, not a replayed trace), separate kernels otherwise. */
+ * pair draws, not a replayed trace), separate kernels otherwise, and where they
+ * are the faster side (states that gather with 3 or 4 column blocks per iteration
+ * of whole views, or of geometric cells on larger problems). */
 bsgd_status bsgd_state_set_split(bsgd_state *s, int split);
 bsgd_status bsgd_state_read_profile(bsgd_state *s, bsgd_profile *out, void *stream);
 

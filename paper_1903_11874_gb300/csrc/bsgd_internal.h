@@ -210,6 +210,7 @@ bool slice_bp_pays(const bsgd_geometry *g, int rows, int views);
 bsgd_status launch_bp_slice(const bsgd_geometry *g, const PlainLaunch &L, const void *r, bsgd_dtype rt,
                             float *x, float scale, int accumulate, cudaStream_t st);
 size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells);
+bool column_solve_apart(const bsgd_geometry *g, int kM, int kN, int cells);
 bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const void *r,
                              bsgd_dtype rt, float *x, float scale, int accumulate, float *w,
                              cudaStream_t st, int per = 64);

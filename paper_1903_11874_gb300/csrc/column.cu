@@ -379,6 +379,20 @@ size_t column_weights_len(const bsgd_geometry *g, int n_rb) {
     return n < (1ull << 32) ? n : 0;
 }
 
+// Whether a gathering state takes FP, residual and weights as passes of their own
+// and not as one: the one holds up to four blocks' rays through its walks (63
+// registers against 40, 8 CTAs per SM against 12), but sets a pixel up once and
+// skips the pass over the bands, which shows where cells leave few rays to walk. us
+// per iteration one / apart, 256^2 x 32 from 45 views, 2, 3, 4 blocks: whole views
+// 735 / 720, 1146 / 1047, 1494 / 1349, geometric cells 485 / 502, 746 / 721, 972 /
+// 921, uniform cells 377 / 411, 566 / 579, 735 / 732; from 11 views, whole views 295
+// / 298, 438 / 423, 566 / 536; 128^2 x 32 from 90 views, 2, 3, 4 blocks, whole views
+// 392 / 406, 592 / 576, 772 / 734, geometric cells 252 / 282, 374 / 390, 482 / 488.
+bool column_solve_apart(const bsgd_geometry *g, int kM, int kN, int cells) {
+    const int64_t work = (int64_t)g->desc.nx * g->desc.ny * (g->desc.nz / g->N) * kN * g->max_views * kM;
+    return kN >= 3 && (cells == BSGD_CELLS_NONE || (cells == BSGD_CELLS_GEOMETRIC && work >= 250000000));
+}
+
 int column_blocks_within(const bsgd_geometry *g, int n_rb, size_t floats) {
     int n = std::min(n_rb, 64);
     while (n > 0 && (column_weights_len(g, n) == 0 || column_weights_len(g, n) > floats)) --n;

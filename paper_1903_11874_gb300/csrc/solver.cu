@@ -10,7 +10,8 @@
 //   update_kernel     x_J += mu g_J
 // With one to four column blocks per iteration the three passes in between are
 // one kernel (siddon.cu), or, where the BP gathers (column.cu), an FP with the
-// residual that leaves the weights r_R - r~^J_R and the gather.
+// residual that leaves the weights r_R - r~^J_R and the gather (three and four
+// blocks mostly take the passes apart then: column_solve_apart).
 // The snapshot r~^J equals keeping Algorithm 1's memory g-hat^i: it stores the
 // residual the last BP of (i, J) used, so the BP of the change replaces
 // g-hat^i_J by the new one exactly.
@@ -1749,7 +1750,8 @@ static bsgd_status one_iteration(bsgd_state *s, void *x, cudaStream_t st, bool d
     // every drawn column block (uniform draws, not a replayed trace)
     const bool replaying = s->replay && k >= s->replay_start && k < s->replay_start + s->replay_n;
     const bool fuse_multi = !s->fused && s->kN <= kMaxFusedCols &&
-                            s->p.pair_sampling == BSGD_PAIRS_UNIFORM && !replaying;
+                            s->p.pair_sampling == BSGD_PAIRS_UNIFORM && !replaying &&
+                            !(s->w && column_solve_apart(g, s->kM, s->kN, s->p.cells));
     const int cols = replaying ? std::min(s->P, g->N) : s->kN;   // distinct blocks, at most
     if (s->max_tiles > 0 && s->fused && !s->split) {
         // one column block per iteration: FP, residual and BP in one pass (column

@@ -288,3 +288,25 @@ def test_sharded_steps(two_blocks, cells):
             for st, x in zip(states, xs):
                 st.shard_end(x, total)
         check_against_oracle(states[0], sum(xs[1:], xs[0].clone()), ost, 1e-5)
+
+
+@pytest.mark.parametrize("kN,cells,apart", [(2, "none", False), (3, "none", True), (4, "none", True),
+                                            (3, "uniform", False), (4, "geometric", False)])
+def test_blocks_that_take_separate_passes(kN, cells, apart):
+    """The rule on one pass or separate ones (three and four blocks): either gives
+    the oracle's image."""
+    s = solve_geometry(kN, nx=96, ny=94, nz=32 * kN, n_views=20, M=2, N=kN, nu=95, nv=95, du=2.2, dv=2.2)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    y = scan(og, s)
+    n_cells = 1 if cells == "none" else 4
+    prm = B.SolveParams(alpha=1.0, gamma=1.0, step_rule=B.STEP_FIXED, mu=2e-5, seed=5, cells=KINDS[cells],
+                        n_cells=n_cells)
+    st = B.State(gg, prm, torch.from_numpy(y).to(DEV))
+    x = torch.zeros(gg.n_cols, device=DEV)
+    st.profile(True)
+    st.block_step(x, 3)
+    prof = st.read_profile()
+    assert (prof["fp"]["launches"], prof["fpbp"]["launches"]) == ((3, 0) if apart else (0, 3))
+    ost = OB.bsgd(og, y.astype(np.float64), OB.Params(2, kN, 1.0, 1.0, 2e-5, seed=5, cells=cells, n_cells=n_cells), 3)
+    check_against_oracle(st, x, ost, 1e-5)
+    assert "solve_gather_kernel" in kernels_of(lambda: st.block_step(x, 1))
