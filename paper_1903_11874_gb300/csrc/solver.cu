@@ -1667,8 +1667,8 @@ size_t state_bytes(const bsgd_geometry_desc &d, int M, int N, const bsgd_solve_p
 // xT = transpose(x): the caller's image is the one to trust at the start of
 // every call (and after the TV prox rewrites it).
 static bsgd_status sync_xT(bsgd_state *s, void *x, cudaStream_t st) {
-    const bsgd_geometry *g = s->g;
     if (!s->xT) return BSGD_OK;
+    const bsgd_geometry *g = s->g;
     const int tiles = ((g->desc.nx + 31) / 32) * ((g->desc.ny + 31) / 32) * g->desc.nz;
     const int gb = std::max(1, std::min(tiles, 152 * 8));
     if (s->st == BSGD_F32) transpose_kernel<float><<<gb, 256, 0, st>>>(g->dg, (const float *)x, (float *)s->xT);
@@ -1924,8 +1924,7 @@ extern "C" bsgd_status bsgd_shard_begin(bsgd_state *s, void *x, float *exchange,
     fill_sample_args(s, A, k);
     sample_kernel<<<1, kSampleThreads, 0, st>>>(A);
     BSGD_CUDA(cudaGetLastError());
-    if (s->max_tiles > 0)
-        BSGD_TRY(launch_fp_solve(g, s->dev, x, s->st, s->P, s->max_tiles, false, st));
+    if (s->max_tiles > 0) BSGD_TRY(launch_fp_solve(g, s->dev, x, s->st, s->P, s->max_tiles, false, st));
     dim3 grid((g->desc.nv + kResRows - 1) / kResRows, g->max_views, s->kM);
     if (s->st == BSGD_F32) shard_partial_kernel<float><<<grid, 256, 0, st>>>(g->dg, s->dev, exchange);
     else if (s->st == BSGD_BF16) shard_partial_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->dg, s->dev, exchange);
