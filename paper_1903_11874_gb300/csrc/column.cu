@@ -210,26 +210,30 @@ __device__ __forceinline__ void slice_view(const DeviceGeom &G, int a, int xx, i
 // Back projection of a 2D kind into rows [y0, y1) of the image, as a gather: a
 // CTA takes 32 pixels of a row, its 8 warps every 8th view each, whichever row
 // block it is of; a thread tests the detector columns whose shadow its pixel is
-// in (one to three) and adds
-// weight x chord. 256^2 pixels from 360 fan views of 384 bins (30 M updates): 193
-// us as a scatter, whose atomics meet on 65536 addresses, 136 us gathered (168 us
-// with the lines as 32-byte records: a warp's load then spans ten 128-byte
-// lines). What bounds it: issue slots, half of them for finding the columns, and
-// lanes that wait for the ones with three columns.
-// kMany: the views of several row blocks, listed on chip 256 at a time (dealt
-// block by block, blocks of one view leave seven warps idle: 64^2 from 90 blocks
-// 94 us, listed 21, scattered 23; 512^2 from 80 blocks of 9 views 1171, 995, 977).
-// One block reads its views in place (256^2 as above 133 us, listed 144).
-template <bool kParallel, bool kMany, typename T>
-__global__ void __launch_bounds__(256) bp_slice_kernel(const DeviceGeom G, const RowSel R, int y0,
-                                                       const T *__restrict__ r, float scale,
-                                                       float *__restrict__ x, int add) {
+// in (one to three) and adds weight x chord. 256^2 pixels from 360 fan views of 384
+// bins (30 M updates): 193 us as a scatter, whose atomics meet on 65536 addresses,
+// 127 us gathered (168 us with the lines as 32-byte records: a warp's load then
+// spans ten 128-byte lines). What bounds it: issue slots, half of them for finding
+// the columns, and lanes that wait for the ones with three columns.
+// kViews: all of the geometry's in order; the listed blocks', listed on chip 256 at a
+// time; or block by block, read in place, where a block's views fill the warps (blocks
+// of 64 views or more: 512^2 from three of 90, 351 us, listed 359). Small blocks leave
+// warps idle: 64^2 from 90 blocks of one view 94 us block by block, 11 in order, 23
+// scattered; 512^2 from 80 blocks of 9 views 1171, 894, 977; 15 of 360 blocks of one
+// view into 256^2 31, listed 18, scattered 35. 32 registers, so that 8 CTAs are
+// resident (36: 4 % slower, 1024^2 from one view 39 us for 29); the blocks' form has
+// them by itself, and loses 2 % where it is told to.
+enum SliceViews { kSliceAll, kSliceListed, kSliceBlocks };
+
+template <bool kParallel, SliceViews kViews, typename T>
+__device__ __forceinline__ void slice_body(const DeviceGeom &G, const RowSel &R, int y0, const T *__restrict__ r,
+                                           float scale, float *__restrict__ x, int add) {
     __shared__ float s[8][32];
     const int tiles = (G.nx + 31) / 32, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int xx = (int)(blockIdx.x % tiles) * 32 + lane, y = y0 + (int)(blockIdx.x / tiles);
     const float fx = (float)xx - 0.5f * (float)G.nx, fy = (float)y - 0.5f * (float)G.ny;
     float acc = 0.f;
-    if (kMany) {
+    if (kViews == kSliceListed) {
         __shared__ int s_views[256];
         const int slots = R.n * G.max_views;
         for (int b = 0; b < slots; b += 256) {
@@ -240,6 +244,8 @@ __global__ void __launch_bounds__(256) bp_slice_kernel(const DeviceGeom G, const
                 if (s_views[q] >= 0)   // (a block with fewer views than the largest)
                     slice_view<kParallel>(G, s_views[q], xx, y, fx, fy, r, scale, acc);
         }
+    } else if (kViews == kSliceAll) {
+        for (int a = warp; a < G.n_views; a += 8) slice_view<kParallel>(G, a, xx, y, fx, fy, r, scale, acc);
     } else {
         for (int k = 0; k < R.n; ++k) {
             const int *views = G.block_views + R.ids[k] * G.max_views;
@@ -254,6 +260,20 @@ __global__ void __launch_bounds__(256) bp_slice_kernel(const DeviceGeom G, const
     for (int q = 1; q < 8; ++q) acc += s[q][lane];
     float *p = x + (int64_t)y * G.nx + xx;
     *p = add ? *p + acc : acc;
+}
+
+template <bool kParallel, SliceViews kViews, typename T>
+__global__ void __launch_bounds__(256, 8) bp_slice_kernel(const DeviceGeom G, const RowSel R, int y0,
+                                                          const T *__restrict__ r, float scale,
+                                                          float *__restrict__ x, int add) {
+    slice_body<kParallel, kViews>(G, R, y0, r, scale, x, add);
+}
+
+template <bool kParallel, typename T>
+__global__ void __launch_bounds__(256) bp_slice_blocks_kernel(const DeviceGeom G, const RowSel R, int y0,
+                                                              const T *__restrict__ r, float scale,
+                                                              float *__restrict__ x, int add) {
+    slice_body<kParallel, kSliceBlocks>(G, R, y0, r, scale, x, add);
 }
 
 }  // namespace
@@ -457,21 +477,27 @@ bsgd_status launch_bp_slice(const bsgd_geometry *g, const PlainLaunch &L, const 
                             float *x, float scale, int accumulate, cudaStream_t st) {
     const int y0 = g->plane_start[L.j0], y1 = g->plane_start[L.j1];
     const unsigned grid = (unsigned)((g->desc.nx + 31) / 32) * (y1 - y0);
-    for (int k = 0; k < L.n_rb; k += 64) {
+    // all blocks: one launch, whose view order does not read the list
+    const bool all = L.n_rb == g->M;
+    for (int k = 0; k < L.n_rb; k += all ? L.n_rb : 64) {
         RowSel R{};
         R.n = std::min(64, L.n_rb - k);
         for (int t = 0; t < R.n; ++t) R.ids[t] = L.row_ids[k + t];
         const int add = accumulate || k > 0;
-#define SLICE_GO2(T, MANY)                                                                                     \
+#define SLICE_KIND(KERNEL, ...)                                                                                \
     if (g->desc.kind == BSGD_PAR2D)                                                                            \
-        bp_slice_kernel<true, MANY, T><<<grid, 256, 0, st>>>(g->dg, R, y0, (const T *)r, scale, x, add);       \
-    else bp_slice_kernel<false, MANY, T><<<grid, 256, 0, st>>>(g->dg, R, y0, (const T *)r, scale, x, add);
-#define SLICE_GO(T) if (R.n > 1) { SLICE_GO2(T, true) } else { SLICE_GO2(T, false) }
+        KERNEL<true, __VA_ARGS__><<<grid, 256, 0, st>>>(g->dg, R, y0, rr, scale, x, add);                      \
+    else KERNEL<false, __VA_ARGS__><<<grid, 256, 0, st>>>(g->dg, R, y0, rr, scale, x, add);
+#define SLICE_GO(T)                                                                                            \
+    const T *rr = (const T *)r;                                                                                \
+    if (all) { SLICE_KIND(bp_slice_kernel, kSliceAll, T) }                                                     \
+    else if (R.n > 1 && g->max_views < 64) { SLICE_KIND(bp_slice_kernel, kSliceListed, T) }                    \
+    else { SLICE_KIND(bp_slice_blocks_kernel, T) }
         if (rt == BSGD_F32) { SLICE_GO(float) }
         else if (rt == BSGD_BF16) { SLICE_GO(__nv_bfloat16) }
         else { SLICE_GO(__half) }
 #undef SLICE_GO
-#undef SLICE_GO2
+#undef SLICE_KIND
         BSGD_CUDA(cudaGetLastError());
     }
     return BSGD_OK;

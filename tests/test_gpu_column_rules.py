@@ -43,6 +43,21 @@ def test_slice_views_dealt_over_all_blocks(views, M, block):
     assert torch.equal(again, got)
 
 
+@pytest.mark.parametrize("views,M,pick", [(90, 45, range(0, 45, 2)), (300, 3, [2, 0]), (140, 70, range(67)),
+                                          (29, 4, [1, 3])])
+def test_slice_of_some_blocks(views, M, pick):
+    """Blocks chosen by the caller: small ones listed, large ones one after another,
+    more than a launch takes, uneven ones (the bound of the plain gather's tests)."""
+    s = fan(70, views, 97, M, np.arange(views) % M)
+    og, gg = oracle_geom(s), gpu_geom(s)
+    r = synth.normal_array(views * 97, 3).astype(np.float32)
+    x = torch.full((70 * 70,), 2.0, device=DEV)
+    B.bsgd_back_project(gg, torch.from_numpy(r).to(DEV), x, row_blocks=list(pick))
+    rows = np.sort(np.concatenate([P.rows_of_views(og, P.row_block_views(og, M, i)) for i in pick]))
+    ref = P.bp_rows(og, r.astype(np.float64)[rows], rows, None)
+    assert rel_l2(x.cpu().double().numpy(), ref.reshape(-1)) <= 4e-5
+
+
 FAR = {
     "cone_3e5": dict(kind="cone3d", nx=64, ny=64, nz=40, dx=1.0, dy=1.0, dz=1.0, n_views=6, nu=70, nv=45, du=2.0,
                      dv=2.0, dso=3e5, dsd=6e5),
