@@ -91,14 +91,14 @@ __global__ void __launch_bounds__(256) column_weights_kernel(const DeviceGeom G,
 
 // The columns of a CTA: kGatherAcross along x, kGatherRows along y, one per warp.
 // out(index, value) for every voxel of planes [z0, z1), along x.
-template <class View, class Out>
+template <bool kNear, class View, class Out>
 __device__ __forceinline__ void gather_cta(const DeviceGeom &G, int n_slots, View &&view, const float *__restrict__ w,
                                            int z0, int z1, int n_cells, Out &&out) {
     __shared__ GatherWarp warps[kGatherWarps];
     const int tiles = (G.nx + kGatherAcross - 1) / kGatherAcross;
     const int x0 = blockIdx.x % tiles * kGatherAcross, y0 = blockIdx.x / tiles * kGatherRows;
     const int warp = threadIdx.x >> 5, x = x0 + warp % kGatherAcross, y = y0 + warp / kGatherAcross;
-    if (x < G.nx && y < G.ny) gather_column(G, n_slots, view, w, x, y, z0, z1, n_cells, warps[warp]);
+    if (x < G.nx && y < G.ny) gather_column<kNear>(G, n_slots, view, w, x, y, z0, z1, n_cells, warps[warp]);
     __syncthreads();
     for (int k = threadIdx.x; k < (z1 - z0) * kGatherWarps; k += blockDim.x) {
         const int c = k % kGatherWarps, z = k / kGatherWarps, xx = x0 + c % kGatherAcross, yy = y0 + c / kGatherAcross;
@@ -109,17 +109,19 @@ __device__ __forceinline__ void gather_cta(const DeviceGeom &G, int n_slots, Vie
 
 // x = (or +=) the plain back projection of planes [z0, z1), kGatherChunks chunks
 // of 32 per CTA (grid y).
+template <bool kNear>
 __global__ void __launch_bounds__(32 * kGatherWarps, 4)
     bp_gather_kernel(const DeviceGeom G, const RowSel R, int z0, int z1, const float *__restrict__ w,
                      float *__restrict__ x, int add) {
     auto view = [&](int &slot, int &) { return gather_view(G, R, slot); };
     const int zb = z0 + (int)blockIdx.y * 32 * kGatherChunks;
-    gather_cta(G, gather_slots(G, R), view, w, zb, min(z1, zb + 32 * kGatherChunks), 1,
+    gather_cta<kNear>(G, gather_slots(G, R), view, w, zb, min(z1, zb + 32 * kGatherChunks), 1,
                [&](int64_t k, float v) { x[k] = add ? x[k] + v : v; });
 }
 
 // g_J += (A_R^J)^T w over the drawn pairs of column block J (blockIdx.z of the
 // iteration's blocks).
+template <bool kNear>
 __global__ void __launch_bounds__(32 * kGatherWarps, 4) solve_gather_kernel(const DeviceGeom G, const SolveDev S) {
     __shared__ int s_pairs[kMaxPairs];
     const Work &W = *S.work;
@@ -141,7 +143,7 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 4) solve_gather_kernel(cons
         if (S.n_cells > 1) cell = S.cells[slot];
         return G.block_views[W.pair_i[p] * G.max_views + s];
     };
-    gather_cta(G, np * G.max_views, view, S.w, zb, min(z1, zb + 32 * kGatherChunks), S.n_cells,
+    gather_cta<kNear>(G, np * G.max_views, view, S.w, zb, min(z1, zb + 32 * kGatherChunks), S.n_cells,
                [&](int64_t k, float v) { S.g[k] += v; });
 }
 
@@ -419,6 +421,10 @@ int column_blocks_within(const bsgd_geometry *g, int n_rb, size_t floats) {
     return n;
 }
 
+// Whether a chunk on both sides of the source's height would be widened by more than
+// a row (gather_column).
+static bool gather_near(const bsgd_geometry *g) { return g->dg.vslack > 1.f; }
+
 static dim3 gather_grid(const bsgd_geometry *g, int planes, int z) {
     const int across = (g->desc.nx + kGatherAcross - 1) / kGatherAcross, rows = (g->desc.ny + kGatherRows - 1) / kGatherRows;
     return dim3((unsigned)(across * rows), (planes + 32 * kGatherChunks - 1) / (32 * kGatherChunks), z);
@@ -437,7 +443,8 @@ bsgd_status launch_bp_column(const bsgd_geometry *g, const PlainLaunch &L, const
         if (rt == BSGD_F32) column_weights_kernel<float><<<wg, 256, 0, st>>>(g->dg, R, L.j0, L.j1, (const float *)r, scale, w);
         else if (rt == BSGD_BF16) column_weights_kernel<__nv_bfloat16><<<wg, 256, 0, st>>>(g->dg, R, L.j0, L.j1, (const __nv_bfloat16 *)r, scale, w);
         else column_weights_kernel<__half><<<wg, 256, 0, st>>>(g->dg, R, L.j0, L.j1, (const __half *)r, scale, w);
-        bp_gather_kernel<<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, R, z0, z1, w, x, accumulate || k > 0);
+        if (gather_near(g)) bp_gather_kernel<true><<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, R, z0, z1, w, x, accumulate || k > 0);
+        else bp_gather_kernel<false><<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, R, z0, z1, w, x, accumulate || k > 0);
         BSGD_CUDA(cudaGetLastError());
     }
     return BSGD_OK;
@@ -516,7 +523,9 @@ bsgd_status launch_column_change(const bsgd_geometry *g, const SolveDev &S, bsgd
 bsgd_status launch_column_solve(const bsgd_geometry *g, const SolveDev &S, int max_cols, cudaStream_t st) {
     int planes = 1;
     for (int j = 0; j < g->N; ++j) planes = std::max(planes, g->plane_start[j + 1] - g->plane_start[j]);
-    solve_gather_kernel<<<gather_grid(g, planes, max_cols), 32 * kGatherWarps, 0, st>>>(g->dg, S);
+    const dim3 grid = gather_grid(g, planes, max_cols);
+    if (gather_near(g)) solve_gather_kernel<true><<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, S);
+    else solve_gather_kernel<false><<<grid, 32 * kGatherWarps, 0, st>>>(g->dg, S);
     BSGD_CUDA(cudaGetLastError());
     return BSGD_OK;
 }

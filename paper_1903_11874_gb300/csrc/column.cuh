@@ -167,16 +167,16 @@ struct GatherVoxel {
 // magic bits, t0 ds, dt ds, rows per voxel of height at the window's low end},
 // `skip` rows above the window's first. The rows of weights are padded by what a
 // chunk of planes can reach past the detector's edges.
-// kMiddle: the chunk holds a voxel that needs the middle's form, or lies on both
-// sides of the source's height with a large slack (gather_middle). Below that, a
-// window's low end is where the ray enters the cell, and A.w is of where it leaves
-// it: its rows per voxel are worked out again.
-template <bool kMiddle>
+// kMiddle: the chunk holds a voxel that needs the middle's form. kNear: it lies on
+// both sides of the source's height, too, and takes no slack (gather_column): below
+// that height, a window's low end is where the ray enters the cell, and A.w is of
+// where it leaves it, so that its rows per voxel are worked out again.
+template <bool kMiddle, bool kNear = false>
 __device__ __forceinline__ void gather_pair(const GatherVoxel &V, float skip, const float4 &A,
                                             const float *__restrict__ w, float &acc) {
     const float t1 = A.y + A.z;
     // first row above the window's low end: floor + 1
-    const float c = kMiddle && V.klo < 0.f ? __fdividef(1.f, A.y) : A.w;
+    const float c = kNear && V.klo < 0.f ? __fdividef(1.f, A.y) : A.w;
     const float S = __fadd_rd(fmaf(V.klo, c, V.vlow), kMagic + 1.f + skip);
     const float *__restrict__ row = w + (__float_as_uint(A.x) + __float_as_uint(S));
     const float w0 = __ldg(row), w1 = __ldg(row + 1);
@@ -194,14 +194,9 @@ __device__ __forceinline__ void gather_pair(const GatherVoxel &V, float skip, co
 }
 
 // Whether a chunk holds a voxel that needs the middle's form: the source's height
-// lies inside it, or a level row of rays in its lower face. A chunk on both sides
-// of the source's height that holds neither has its windows widened by G.vslack, a
-// bound for the cell nearest to the source, which costs a pair of rows per two rows
-// of it, everywhere. Above a row it takes the middle's form, too: 128^2 x 32 from 60
-// views with the source 20 voxels from the volume (17 rows) 130 us against 413, 60
-// voxels (2.4 rows) 109 against 130; widened by 0.27 row, 250^3 takes 4 % less.
+// lies inside it, or a level row of rays in its lower face.
 __device__ __forceinline__ bool gather_middle(const DeviceGeom &G, float ka, float kb) {
-    return kb > 0.f && ka <= 0.f && ((G.nv & 1) || G.zs != floorf(G.zs) || (ka < 0.f && G.vslack > 1.f));
+    return kb > 0.f && ka <= 0.f && ((G.nv & 1) || G.zs != floorf(G.zs));
 }
 
 // Rows that a chunk of planes with faces ka, kb (heights) can meet in a
@@ -228,7 +223,13 @@ __device__ __forceinline__ bool gather_window(const DeviceGeom &G, const float4 
 // chunks of 32). The sum of plane z0 + 32 q + lane is left at sums[q][lane].
 // view(slot, cell): the view (-1: none); sets its slot among the weights and its
 // drawn detector cell (-1: all).
-template <class View>
+// A chunk on both sides of the source's height has its windows widened by G.vslack, a
+// bound for the cell nearest to the source, which costs a pair of rows per two rows of
+// it, everywhere. kNear, taken above a row: planes below that height find their windows
+// by themselves. 128^2 x 32 from 60 views with the source 20 voxels from the volume (17
+// rows) 133 us against 413, x 48 with 60 voxels (2.4 rows) 167 against 184; where the
+// bound is small the reciprocal costs 2 to 4 %, and a choice inside the loop 30 %.
+template <bool kNear, class View>
 __device__ __forceinline__ void gather_column(const DeviceGeom &G, int n_slots, View &&view,
                                               const float *__restrict__ w, int x, int y, int z0, int z1,
                                               int n_cells, GatherWarp &M) {
@@ -247,12 +248,13 @@ __device__ __forceinline__ void gather_column(const DeviceGeom &G, int n_slots, 
         for (int q = 0; q < chunks; ++q) {
             const int zb = z0 + 32 * q, planes = min(32, z1 - zb);
             const float ka = (float)zb - G.zs, kb = ka + (float)planes;
-            const bool middle = gather_middle(G, ka, kb);
-            const float slack = ka < 0.f && kb > 0.f && !middle ? G.vslack : 0.f;
+            const bool both = ka < 0.f && kb > 0.f;
+            const float slack = !kNear && both ? G.vslack : 0.f;
             int extra = 0;
             bool hit = have && gather_window(G, E, ka, kb, slack, half, E.w, extra);
             unsigned m = __ballot_sync(0xffffffffu, hit);
             if (!m) continue;
+            const bool middle = gather_middle(G, ka, kb) || (kNear && both);
             const GatherVoxel V(G, zb + min(lane, planes - 1), slack);
             float acc = M.sums[q][lane];
             for (float skip = 0.f; m; skip += 2.f) {
@@ -264,7 +266,7 @@ __device__ __forceinline__ void gather_column(const DeviceGeom &G, int n_slots, 
                 if (middle) {
                     for (int e = 0; e < n; ++e) {
                         const float4 A = M.work[e];
-                        gather_pair<true>(V, skip, A, w, acc);
+                        gather_pair<true, kNear>(V, skip, A, w, acc);
                         if (V.centre && skip == 0.f)   // the level row, stored as row 1 of its side
                             acc = fmaf(A.z, __ldg(w + (__float_as_uint(A.x) + (uint32_t)(kMagicBits + (G.nv >> 1)))), acc);
                     }
