@@ -40,19 +40,23 @@ WORKLOAD = ("cone3d 256^3 (1 mm), 360 views / 360 deg, 256x256 det (1.6 mm), DSO
             "pairs; step = 1 epoch = 64 block iterations")
 METRIC = "GVox-ray updates/s (FP+BP)"
 UNIT = "GVox-ray/s"
-# FP32-pipe instructions every Siddon update needs at the least: two minima for
-# the next crossing, the segment difference, the accumulate / weight product and
-# the recomputed crossing.
+# FP32-pipe instructions that an update of the incremental Siddon walk needs at
+# the least: two minima for the next crossing, the segment difference, the
+# accumulate / weight product and the recomputed crossing. The gathering BP finds
+# its crossings otherwise; its updates are counted at the walk's cost.
 ALU_OPS_PER_UPDATE = 5
 # DRAM bytes (read + write) per pass, from an ncu capture of the current kernels;
-# null for passes that were not captured (the FP with the residual and the
-# gathering BP that now make up the fused pass).
+# null for passes that were not captured as a whole (the fused pass is the FP with
+# the residual and the gathering BP).
 TRAFFIC_PER_LAUNCH = {}
 # What binds the passes on chip, from ncu captures of the current kernels
-# (summarised under profiles/): the gathering BP on one slab of this workload.
-ON_CHIP_NCU = {"fpbp": {"kernel": "bp_gather_kernel (the BP's half of the pass)", "l1tex_pct": 75.9,
-                        "issue_active_pct": 66.9, "warp_instructions_per_launch": 161_189_658,
-                        "updates_per_launch": 171_855_901}}
+# (summarised under profiles/): each half of the pass by itself.
+ON_CHIP_NCU = {"fpbp": {
+    "fp": {"kernel": "fpbp_solve_kernel<float, true>, one pair of this workload", "l1tex_pct": 61.0,
+           "issue_active_pct": 61.1, "warp_instructions_per_launch": 130_521_796},
+    "bp": {"kernel": "bp_gather_kernel, 45 views into one 32-plane slab of this workload by a plain back projection",
+           "l1tex_pct": 75.9, "issue_active_pct": 66.9, "warp_instructions_per_launch": 161_189_658,
+           "updates_per_launch": 171_855_901}}}
 
 
 # Serving workload: Poisson arrivals (20 / s), request sizes n^3 with (256 / n) mm
@@ -326,7 +330,7 @@ def run_cuda(args):
     roofline = {
         "bound": "alu", "kernel": "fpbp_solve_kernel + solve_gather_kernel" if dom == "fpbp" else "%s_solve_kernel" % dom,
         "achieved": round(achieved, 3), "peak": round(alu_peak, 2),
-        "unit": "T FP32-pipe instr/s (%d per update)" % ALU_OPS_PER_UPDATE,
+        "unit": "T FP32-pipe instr/s (%d per update, the Siddon walk's)" % ALU_OPS_PER_UPDATE,
         "frac": round(achieved / alu_peak, 4), "traffic": TRAFFIC_PER_LAUNCH.get(dom),
         "peak_source": "152 SMs x 128 FP32 lanes x %.0f MHz (max SM clock)" % sm_max,
         "launch_ms": round(launch_ms, 4), "updates_per_launch": int(upd_per_launch),

@@ -151,17 +151,20 @@ bsgd_status bsgd_forward_project(const bsgd_geometry *g, const void *x, bsgd_dty
                                  int accumulate, int batch, void *stream);
 
 /*
- * Back projection x_B (= or +=) scale * (A_S^B)^T r_S, the exact transpose of
- * bsgd_forward_project (Algorithm 1's BP step).
+ * Back projection x_B (= or +=) scale * (A_S^B)^T r_S, the transpose of
+ * bsgd_forward_project (Algorithm 1's BP step; exact where it scatters, to float
+ * rounding of the rays' crossings where it gathers).
  *  r: device, batch * n_rows elements of type rt; rows outside the selected
  *     row blocks are not read.
  *  x: device, batch * n_cols float32 (BSGD_F32 only: the sums are kept in
  *     float). With accumulate = 0 the voxels of the selected
  *     column blocks are cleared first; other voxels are untouched.
  * 2D images of 4096 pixels or more gather (the same sum in every run). Larger
- * cone-beam volumes do so too, from weights that the call lays out in the
- * library's memory pool: n_views of the row blocks (at
- * most 64 blocks at a time) * nu * (nv and some padding) floats. Otherwise, or
+ * cone-beam volumes do so too (slabs of 16 planes or more that the detector
+ * covers, sources neither within a few voxels of the volume nor 1e5 voxels from
+ * the detector), from weights that the call lays out in the library's memory
+ * pool: n_views of the row blocks (at most 64 blocks at a time) * nu * (nv and
+ * some padding) floats. Otherwise, or
  * if the pool has no room, the rays scatter: not bit-reproducible run to run
  * (atomic order), results agree to float rounding; the views whose rays run
  * mostly along x then scatter into a y-fastest float32 accumulator from the pool
@@ -334,7 +337,8 @@ typedef struct {
  * A cone-beam state with slabs of 28 planes or more and enough voxels and views
  * per iteration back-projects by gathering (see bsgd_back_project): it then
  * holds the weights of an iteration's pairs (pairs * views per row block * nu *
- * (nv and some padding) floats) in place of a y-fastest accumulator.
+ * (nv and some padding) floats) in place of a y-fastest accumulator, if there is
+ * room for them beside the rest.
  * Errors: INVALID_ARG (alpha, gamma outside (0, 1], residual pair sampling with
  * more than one pair per iteration, n_cells not 2 (2D) or 4 (3D) with cells),
  * OOM, CUDA.

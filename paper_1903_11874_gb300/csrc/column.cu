@@ -473,9 +473,9 @@ size_t column_solve_len(const bsgd_geometry *g, int kM, int kN, bool cells) {
 }
 
 // Whether the back projection of a 2D kind into `rows` image rows gathers: us
-// scattered / gathered, 64^2 from 90 views 15.4 / 14.4, 128^2 from 60 17.4 /
-// 10.5, 100 x 17 of a strip from 180 20.1 / 20.1, 512^2 from 720 930 / 865.
-// Below 4096 pixels the two are level.
+// scattered / gathered, 64^2 from 90 views 15.4 / 10.7, 128^2 from 60 17.4 /
+// 10.5, 100 x 17 of a strip from 180 20.1 / 20.1, 512^2 from 720 977 / 894.
+// At strips of some 2000 pixels the two are level.
 bool slice_bp_pays(const bsgd_geometry *g, int rows, int views) {
     return g->dg.sx && (int64_t)g->desc.nx * rows >= 4096 && views >= 1;
 }
